@@ -65,9 +65,9 @@ struct AFric { float adt, s2, k; int mode; };
 
 __device__ __forceinline__ AFric a_friction(const ANode& C, const SweepConst& K) {
     AFric F{0.f, 0.f, 0.f, 0};
-    if (K.dt_gn2 > 0.f) {
+    if (K.fric) {
         float ex;
-        F.k = fric_k(C.w, C.t, C.e + C.d, K.dt_gn2, F.s2, ex);
+        F.k = fric_k(C.w, C.t, C.c, K, F.s2, ex);
         F.adt = C.w * F.k;
         F.mode = ex >= 0.f ? 2 : 1;
     }
@@ -287,10 +287,10 @@ __device__ __forceinline__ void a_dstage_adj2(const N2& L, const N2& C, const N2
     float2 dq = fma2(mul2(lq, k2), dQq, mul2(nh, add2(QqL, QqR)));
     float2 s2 = v2(0.f), kf = v2(0.f);
     bool clA = false, clB = false;
-    const bool fric = K.dt_gn2 > 0.f;
+    const bool fric = K.fric != 0;
     if (fric) {
         float2 ex;
-        kf = fric_k2(C.w, C.t, add2(C.e, C.d), K.dt_gn2, s2, ex);
+        kf = fric_k2(C.w, C.t, C.c, K, s2, ex);
         clA = ex.x >= 0.f;
         clB = ex.y >= 0.f;
         const float2 adt = mul2(C.w, kf);
@@ -589,17 +589,17 @@ __global__ void __launch_bounds__(AWARPS * 32, SPH ? 2 : CLIFFS_ADJ_LINE_BLOCKS)
     const int strip = blockIdx.x, l0 = blockIdx.y * ALINES;
     const int p0 = strip * AOUT - AHALO;
     const int pA = p0 + 2 * lane;
-    const SweepConst K{A.hmin, A.dwall, A.half_dt, A.dt_gn2, A.transverse, A.inv_dt2_s1};
+    const SweepConst& K = A.K;
     AMet mb[2];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
         const int p = pA + i;
         mb[i] = AMet{0.f, 0.f, 0.f, 0.f};
         if (DIR == 0) {
-            if (p >= 0 && p < A.npos) mb[i] = AMet{A.xa[p], A.xb[p], A.xk[p], 0.f};
+            if (p >= 0 && p < A.npos) mb[i] = AMet{2.f * A.xa[p], 2.f * A.xb[p], A.xk[p], 0.f};
         } else {
             const float4 q = A.ymet[min(max(p, -MET_PAD), A.npos - 1 + MET_PAD)];
-            mb[i] = AMet{q.x, q.y, q.z, q.w};
+            mb[i] = AMet{2.f * q.x, 2.f * q.y, q.z, -q.w};
         }
     }
     static_assert(ALINES == AWARPS, "one line per warp");
@@ -708,7 +708,7 @@ __global__ void __launch_bounds__(AWARPS * 32) k_adj_xfwd(const StepArgs a, cons
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     const int strip = blockIdx.x, r0 = blockIdx.y * ALINES;
     const int c0 = strip * XOUT - 4, cA = c0 + 2 * lane;
-    const SweepConst K{a.hmin, a.dwall, a.half_dt, a.dt_gn2, a.transverse, a.inv_dt2_s1};
+    const SweepConst& K = a.K;
     const bool colA = cA >= 0 && cA < a.nx, colB = cA + 1 >= 0 && cA + 1 < a.nx;
     float2 il = v2(0.f), ir = v2(0.f), k2 = v2(0.f);
     if (colA) { il.x = a.xa[cA]; ir.x = a.xb[cA]; k2.x = a.xk[cA]; }
@@ -727,7 +727,7 @@ __global__ void __launch_bounds__(AWARPS * 32) k_adj_xfwd(const StepArgs a, cons
         XMet2 m{il, ir, k2};
         if (SPH) {
             const float2 f = v2(a.xrow[r]);
-            m.inv_l = mul2(m.inv_l, f); m.inv_r = mul2(m.inv_r, f); m.k2 = mul2(m.k2, f);
+            m.hl = mul2(m.hl, f); m.hr = mul2(m.hr, f); m.k2 = mul2(m.k2, f);
         }
         unsigned ends = 0u;                         // open outer edges among this lane's columns
         if (OPEN) {
@@ -844,7 +844,7 @@ cudaError_t launch_adj_line(const AdjLineArgs& A, int dir, bool sph, cudaStream_
                                      (const void*)k_adj_line<1, false, true>, (const void*)k_adj_line<1, true, true>};
     AdjLineArgs aa = A;
     void* args[] = {&aa};
-    return launch_pdl(t[(sph ? 1 : 0) + (dir ? 2 : 0) + (A.inv_dt2_s1 > 0.f ? 4 : 0)], grid, dim3(AWARPS * 32),
+    return launch_pdl(t[(sph ? 1 : 0) + (dir ? 2 : 0) + (A.K.inv_dt2 > 0.f ? 4 : 0)], grid, dim3(AWARPS * 32),
                       args, s, pdl);
 }
 
@@ -862,7 +862,7 @@ cudaError_t launch_adj_xfwd(const StepArgs& a, const float* e, const float* u, c
         (const void*)k_adj_xfwd<false, true, true, true>, (const void*)k_adj_xfwd<true, true, true, true>};
     StepArgs aa = a;
     void* args[] = {&aa, (void*)&e, (void*)&u, (void*)&v, &te, &tu, &tv, &tpitch};
-    return launch_pdl(t[(a.sph ? 1 : 0) + (a.dt_gn2 > 0.f ? 2 : 0) + (a.inv_dt2_s1 > 0.f ? 4 : 0) +
+    return launch_pdl(t[(a.sph ? 1 : 0) + (a.K.fric ? 2 : 0) + (a.K.inv_dt2 > 0.f ? 4 : 0) +
                         (a.open_edges ? 8 : 0)],
                       grid, dim3(AWARPS * 32), args, s, pdl);
 }

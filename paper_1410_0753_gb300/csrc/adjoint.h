@@ -17,9 +17,7 @@ struct AdjLineArgs {
     const int* gxy;                  // gauge nodes (ix, iy)
     int G;
     const float* seed;               // dL/d (eta, u, v) at the gauges for this step ([G][3]), or null
-    float hmin, dwall, half_dt, dt_gn2;
-    int transverse;
-    float inv_dt2_s1;                // 1/dt^2 with eq. (solver1), else 0
+    SweepConst K;
     int open_lo, open_hi;            // the line's first / last node is at an open outer edge
 };
 

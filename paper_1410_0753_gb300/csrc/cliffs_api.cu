@@ -96,8 +96,9 @@ __global__ void k_cfl(const double* d64, int nx, int ny, const float* xa, const 
     const double d = d64[i];
     if (!(d > 0.0)) return;
     double inv = 0.0;
-    if (nx > 1) inv = fmax((double)xa[c], (double)xb[c]) * (double)xrow[r];
-    if (ny > 1) inv = fmax(inv, fmax((double)ymet[r].x, (double)ymet[r].y));
+    // the tables hold 1/(2 dx)
+    if (nx > 1) inv = 2.0 * fmax((double)xa[c], (double)xb[c]) * (double)xrow[r];
+    if (ny > 1) inv = fmax(inv, 2.0 * fmax((double)ymet[r].x, (double)ymet[r].y));
     const float cour = (float)(sqrt(9.81 * d) * dt * inv);
     atomicMax(out, __float_as_uint(cour));
 }
@@ -232,6 +233,22 @@ __global__ void k_boundary(const float* nrec, int nnodes, const int* slot, const
     for (int q = 0; q < 3; ++q) vals[(t * 3 + q) * np + p] = acc[q];
 }
 
+// Rows of the fused kernel's windows that hold a node dry at rest (d < h_min) or a permanent
+// wall: hard[strip][row], one warp per row of a window (64 columns from 56 strip).
+__global__ void __launch_bounds__(256) k_hard_rows(const float* d32, int nx, int ny, int pitch, int nstrips, float hmin,
+                                                   float dwall, unsigned char* hard) {
+    const int lane = threadIdx.x & 31;
+    const long long w = blockIdx.x * 8ll + (threadIdx.x >> 5);
+    if (w >= (long long)nstrips * ny) return;
+    const int st = (int)(w / ny), r = (int)(w % ny);
+    bool dry = false;
+    for (int c = st * XOUT + lane; c < min(nx, st * XOUT + XWIN); c += 32) {
+        const float d = d32[(long long)r * pitch + c];
+        dry |= !(d >= hmin) || !(d >= dwall);
+    }
+    if (__any_sync(FULL, dry) && lane == 0) hard[w] = 1;
+}
+
 inline unsigned nblk(long long n, int bs = 256) { return (unsigned)((n + bs - 1) / bs); }
 
 // Boundary input for one step: per edge the series and the two records (k, k+1) to mix
@@ -287,6 +304,7 @@ struct cliffs_grid {
     float* eta[2] = {nullptr, nullptr};
     float* u[2] = {nullptr, nullptr};
     float* v[2] = {nullptr, nullptr};
+    float* st[2] = {nullptr, nullptr};       // the state buffers [3][B][plane]; eta, u, v point into them
     float* d32 = nullptr;
     double* d64 = nullptr;
     double* d64b = nullptr;
@@ -294,6 +312,7 @@ struct cliffs_grid {
     float* smax = nullptr;
     float *xa = nullptr, *xb = nullptr, *xk = nullptr, *xrow = nullptr;
     float4* ymet = nullptr;
+    float4* ymp = nullptr;
     int* err = nullptr;
     long long inject_cycles = 0;             // armed by cliffs_inject_wait_expiry
     long long* limit = nullptr;
@@ -319,8 +338,8 @@ struct cliffs_grid {
     // launch geometry
     int kind = 0;                            // 0 fused 2D, 1 x only, 2 y only
     int S = 32, nstrips = 0, nseg = 0;
-    int S_hard = 32;                         // rows per warp in strips with dry nodes / edges
-    std::vector<unsigned char> hard;         // per strip: dry nodes in its window, or an edge
+    std::vector<unsigned char> hard;         // [nstrips][ny]: dry nodes in the strip's window within 3 rows
+    std::vector<double> strip_cost;          // per strip: the cost of its rows (item_cost)
     std::vector<int4> items;                 // fused kernel work items (strip, r0, r1, 0)
     int4* items_dev = nullptr;
     // timing
@@ -475,22 +494,41 @@ int build_samples(cliffs_grid* g) {
     return CLIFFS_OK;
 }
 
-// Work items of the fused kernel: every strip is cut into segments of S rows, or S_hard
-// rows in strips whose window holds dry nodes or reaches past the domain edge (their warps
-// take the wet/dry correction paths on every row, so shorter segments even out the time
-// the warps of one launch take).
-int set_rows_per_warp(cliffs_grid* g, int S, int S_hard) {
+// Work items of the fused kernel. A row whose window has dry nodes within three rows takes the
+// general path, which costs about SLOW_COST rows of open water; every strip is cut into as
+// many segments as its cost holds S rows of open water, at equal costs, so that the warps of
+// one launch take about the same time. (With strips cut into equal numbers of rows, the warps
+// that cross an island decided the time of the launch: 157 us on a 4096^2 grid with ten
+// islands whose rows outside the islands' windows alone take 121 us.)
+const double SLOW_COST = 2.5;
+
+double strip_row_cost(const cliffs_grid* g, int st, int r) {
+    return g->hard[(size_t)st * g->ny + r] ? SLOW_COST : 1.0;
+}
+
+void cut_items(const cliffs_grid* g, int S, std::vector<int4>& items) {
+    items.clear();
+    for (int st = 0; st < g->nstrips; ++st) {
+        const double cost = g->strip_cost[st];
+        const int nseg = std::max(1, std::min(g->ny, (int)std::ceil(cost / S - 1e-9)));
+        double sum = 0.0;
+        int r0 = 0, cut = 1;
+        for (int r = 0; r < g->ny; ++r) {
+            sum += strip_row_cost(g, st, r);
+            if (r + 1 == g->ny || (cut < nseg && sum >= cost * cut / nseg - 1e-9)) {
+                items.push_back(make_int4(st, r0, r + 1, 0));
+                r0 = r + 1;
+                while (cut < nseg && sum >= cost * cut / nseg - 1e-9) ++cut;
+            }
+        }
+    }
+}
+
+int set_rows_per_warp(cliffs_grid* g, int S) {
     g->S = S;
-    g->S_hard = S_hard;
     g->nseg = (g->ny + S - 1) / S;
     if (g->kind == 0) {
-        g->items.clear();
-        for (int st = 0; st < g->nstrips; ++st) {
-            const int h = g->hard.empty() ? 0 : g->hard[st];
-            const int seg = h ? S_hard : S;
-            for (int r0 = 0; r0 < g->ny; r0 += seg)
-                g->items.push_back(make_int4(st, r0, std::min(r0 + seg, g->ny), 0));
-        }
+        cut_items(g, S, g->items);
         cudaFree(g->items_dev);
         g->items_dev = nullptr;
         CK(cudaMalloc(&g->items_dev, sizeof(int4) * g->items.size()));
@@ -499,15 +537,12 @@ int set_rows_per_warp(cliffs_grid* g, int S, int S_hard) {
     return build_samples(g);
 }
 
-int hard_rows(int S) { return std::max(8, (S * 3 / 4) & ~1); }
-
 // warps of one fused launch with S rows per warp, and the warps resident at once
 long long fused_warps(const cliffs_grid* g, int S) {
-    int nhard = 0;
-    for (int st = 0; st < g->nstrips; ++st) nhard += g->hard.empty() ? 0 : g->hard[st];
-    const int Sh = hard_rows(S);
-    return ((long long)(g->nstrips - nhard) * ((g->ny + S - 1) / S) +
-            (long long)nhard * ((g->ny + Sh - 1) / Sh)) * g->B;
+    long long n = 0;
+    for (int st = 0; st < g->nstrips; ++st)
+        n += std::max(1, std::min(g->ny, (int)std::ceil(g->strip_cost[st] / S - 1e-9)));
+    return n * g->B;
 }
 
 long long resident_warps(const cliffs_grid* g) {
@@ -526,6 +561,22 @@ int wave_rows(const cliffs_grid* g, int waves) {
     return 0;
 }
 
+// Modelled time of a launch of n warps with S rows each, in units of the time a scheduler
+// with its four warps takes per row (0.81 us on the 8192^2 grid): a warp takes S rows and
+// about 3.7 more (rows above and below its own, the first copies); full waves take 1 per row,
+// a last wave of one to four warps per scheduler 0.62, 0.74, 0.86 or 1. Launches a little
+// over full waves find room beside warps that end early (3 %). Against measured times over S on grids
+// of 200^2 to 8192^2 the model's choice is within 5 % of the best (8192^2: 435 us at S = 32,
+// 425 at 64, 429 at 128, 483 at 16; 1024^2: 22.9 at 10, 25.1 at 16, 27.1 at 8; 2048^2
+// geographic: 59.3 at 40, 63.8 at 20, 73.0 at 32).
+double launch_cost(int S, long long n, long long resident, long long nsched) {
+    const double last[5] = {0.0, 0.62, 0.74, 0.86, 1.0};
+    const double x = 0.97 * (double)n / (double)resident;
+    const double full = std::floor(x);
+    const int q = std::min(4, (int)std::ceil((x - full) * (double)resident / (double)nsched));
+    return (S + 3.7) * (full + last[q]);
+}
+
 int choose_geometry(cliffs_grid* g) {
     if (g->ny == 1) {
         g->kind = 1;
@@ -540,19 +591,17 @@ int choose_geometry(cliffs_grid* g) {
     } else {
         g->kind = 0;
         g->nstrips = fused_strips(g->nx);
-        // rows per warp S: each warp walks S + 6 rows (3-row halo above and below), so the
-        // cost of one wave of warps is ~ S + 6; pick the even S minimising waves * (S + 6)
-        // with the resident warps the occupancy calculator reports (ties go to the larger S)
+        // rows per warp S: the one with the smallest modelled time (the larger on a tie)
         const long long resident = resident_warps(g);
+        const long long nsched = std::max<long long>(1, resident / std::max(1, fused_blocks_per_sm(g->cfg.coords != 1)));
         double best = 1e300;
         int bestS = 32;
-        for (int S = 8; S <= 1024; S += (S < 128 ? 2 : 32)) {
-            if (S > 2 * g->ny && S != 8) break;
-            const long long warps = fused_warps(g, S);
-            const double cost = (double)((warps + resident - 1) / resident) * (S + 6);
+        for (int S = 2; S <= 512; S += (S < 16 ? 1 : S < 128 ? 2 : 32)) {
+            if (S > g->ny && S != 2) break;
+            const double cost = launch_cost(S, fused_warps(g, S), resident, nsched);
             if (cost <= best) { best = cost; bestS = S; }
         }
-        return set_rows_per_warp(g, bestS, hard_rows(bestS));
+        return set_rows_per_warp(g, bestS);
     }
     return build_samples(g);
 }
@@ -611,16 +660,16 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
-// a [batch][ny][pitch] FP32 tensor (batch 1 for the depth) read in 64 x 2 x 1 boxes;
-// out-of-range boxes fill with zeros
-int make_map(CUtensorMap* m, const float* base, int rank, int pitch, int ny, int batch) {
+// nf fields of a [batch][ny][pitch] FP32 tensor, fs floats apart, read in 64 x 4 x 1 x nf boxes
+// (nf = 0: one [ny][pitch] plane, 64 x 4 boxes); out-of-range boxes fill with zeros
+int make_map(CUtensorMap* m, const float* base, int pitch, int ny, int batch, long long fs, int nf) {
     auto fn = encode_fn();
     if (!fn) return set_err(CLIFFS_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
-    cuuint64_t dims[3] = {(cuuint64_t)pitch, (cuuint64_t)ny, (cuuint64_t)batch};
-    cuuint64_t strides[2] = {(cuuint64_t)pitch * 4, (cuuint64_t)pitch * ny * 4};
-    cuuint32_t box[3] = {(cuuint32_t)TMA_BOX_COLS, (cuuint32_t)TMA_BOX_ROWS, 1};
-    cuuint32_t es[3] = {1, 1, 1};
-    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, rank, const_cast<float*>(base), dims, strides, box, es,
+    cuuint64_t dims[4] = {(cuuint64_t)pitch, (cuuint64_t)ny, (cuuint64_t)batch, (cuuint64_t)nf};
+    cuuint64_t strides[3] = {(cuuint64_t)pitch * 4, (cuuint64_t)pitch * ny * 4, (cuuint64_t)fs * 4};
+    cuuint32_t box[4] = {(cuuint32_t)TMA_BOX_COLS, (cuuint32_t)TMA_BOX_ROWS, 1, (cuuint32_t)nf};
+    cuuint32_t es[4] = {1, 1, 1, 1};
+    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, nf ? 4 : 2, const_cast<float*>(base), dims, strides, box, es,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return set_err(CLIFFS_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
@@ -628,14 +677,12 @@ int make_map(CUtensorMap* m, const float* base, int rank, int pitch, int ny, int
 }
 
 int make_maps(cliffs_grid* g) {
+    const long long fs = (long long)g->B * g->plane;
     for (int k = 0; k < 2; ++k) {
         StepMaps& M = g->maps[k];
-        int rc = make_map(&M.e, g->eta[k], 3, g->pitch, g->ny, g->B);
-        if (!rc) rc = make_map(&M.u, g->u[k], 3, g->pitch, g->ny, g->B);
-        if (!rc) rc = make_map(&M.v, g->v[k], 3, g->pitch, g->ny, g->B);
-        if (!rc) rc = make_map(&M.d, g->d32, 3, g->pitch, g->ny, 1);
-        if (!rc) rc = make_map(&M.em, g->emax, 3, g->pitch, g->ny, g->B);
-        if (!rc) rc = make_map(&M.sm, g->smax, 3, g->pitch, g->ny, g->B);
+        int rc = make_map(&M.s, g->st[k], g->pitch, g->ny, g->B, fs, 3);
+        if (!rc) rc = make_map(&M.d, g->d32, g->pitch, g->ny, 1, 0, 0);
+        if (!rc) rc = make_map(&M.mw, g->emax, g->pitch, g->ny, g->B, fs, 2);
         if (rc) return rc;
     }
     return CLIFFS_OK;
@@ -643,10 +690,11 @@ int make_maps(cliffs_grid* g) {
 
 void fill_step_args(cliffs_grid* g, StepArgs& a, int in, int out) {
     a.eta_in = g->eta[in]; a.u_in = g->u[in]; a.v_in = g->v[in];
-    a.eta_out = g->eta[out]; a.u_out = g->u[out]; a.v_out = g->v[out];
+    a.eta_out = g->eta[out];
+    a.fs_out = a.fs_max = (long long)g->B * g->plane;
     a.d = g->d32;
-    a.xa = g->xa; a.xb = g->xb; a.xk = g->xk; a.xrow = g->xrow + MET_PAD; a.ymet = g->ymet + MET_PAD;
-    a.emax = nullptr; a.smax = nullptr; a.rec_g = nullptr; a.rec_n = nullptr;
+    a.xa = g->xa; a.xb = g->xb; a.xk = g->xk; a.xrow = g->xrow + MET_PAD; a.ymet = g->ymet + MET_PAD; a.ymp = g->ymp + MET_PAD;
+    a.emax = nullptr; a.rec_g = nullptr; a.rec_n = nullptr;
     a.rec_g_bstride = g->grec_cap * g->G * 3;
     a.samp_ptr = g->samp_ptr; a.samp = g->samp;
     a.limit = g->limit;
@@ -654,16 +702,23 @@ void fill_step_args(cliffs_grid* g, StepArgs& a, int in, int out) {
     a.nx = g->nx; a.ny = g->ny; a.pitch = g->pitch; a.plane = g->plane;
     a.S = g->S; a.nstrips = g->nstrips; a.nseg = g->nseg;
     a.items = g->items_dev; a.nitems = (int)g->items.size();
-    a.hmin = (float)g->cfg.h_min;
-    a.dwall = g->cfg.itopo ? -3.402823466e38f : (float)g->cfg.dwall;
-    a.half_dt = (float)(0.5 * g->cfg.dt);
-    a.dt_gn2 = (float)(g->cfg.dt * 9.81 * g->cfg.manning_n2);
-    a.transverse = g->cfg.transverse ? 1 : 0;
+    const double gn2 = g->cfg.dt * 9.81 * g->cfg.manning_n2;
+    a.K.hmin = (float)g->cfg.h_min;
+    a.K.dwall = g->cfg.itopo ? -3.402823466e38f : (float)g->cfg.dwall;
+    a.K.half_dt = (float)(0.5 * g->cfg.dt);
+    a.K.inv_dt2 = g->cfg.solver == 1 ? (float)(1.0 / (g->cfg.dt * g->cfg.dt)) : 0.f;
+    a.K.fric = (float)gn2 > 0.f;
+    a.K.transverse = g->cfg.transverse ? 1 : 0;
+    a.K.hdt = make_float2(a.K.half_dt, a.K.half_dt);
+    a.K.ntr = g->cfg.transverse ? make_float2(-1.f, -1.f) : make_float2(0.f, 0.f);
+    const float lgf = a.K.fric ? (float)(std::log2(gn2) + 4.0 / 3.0 * std::log2(9.81)) : 0.f;
+    a.K.lgf = make_float2(lgf, lgf);
     a.sph = g->cfg.coords != 1;
     a.wait_cycles = 2000000000LL;            // about a second at the GB300's clocks
     a.tx_pad = 0;
+    a.walls = g->cfg.itopo == 0;
+    fused_ring(false, &a.nslots, &a.slot_floats);
     a.yfirst = 0;
-    a.inv_dt2_s1 = g->cfg.solver == 1 ? (float)(1.0 / (g->cfg.dt * g->cfg.dt)) : 0.f;
     a.open_edges = g->cfg.open_edges;
 }
 
@@ -763,10 +818,10 @@ int input_edges(const cliffs_grid* g) {
 }
 
 void free_grid(cliffs_grid* g) {
-    for (int k = 0; k < 2; ++k) { cudaFree(g->eta[k]); cudaFree(g->u[k]); cudaFree(g->v[k]); }
+    for (int k = 0; k < 2; ++k) cudaFree(g->st[k]);
     cudaFree(g->d32); cudaFree(g->d64); cudaFree(g->d64b);
-    cudaFree(g->emax); cudaFree(g->smax);
-    cudaFree(g->xa); cudaFree(g->xb); cudaFree(g->xk); cudaFree(g->xrow); cudaFree(g->ymet);
+    cudaFree(g->emax);
+    cudaFree(g->xa); cudaFree(g->xb); cudaFree(g->xk); cudaFree(g->xrow); cudaFree(g->ymet); cudaFree(g->ymp);
     cudaFree(g->err); cudaFree(g->limit); cudaFree(g->items_d); cudaFree(g->items_dev);
     cudaFree(g->samp_ptr); cudaFree(g->samp); cudaFree(g->grec); cudaFree(g->nrec);
     cudaFree(g->pt_slot); cudaFree(g->pt_w); cudaFree(g->tmp); cudaFree(g->ured);
@@ -859,19 +914,23 @@ int cliffs_grid_create(const cliffs_config* cfg, cliffs_grid** out) {
     auto fail = [&](int rc) { free_grid(g); return rc; };
     const size_t sb = sizeof(float) * (size_t)g->B * g->plane;
 #define CKG(call) do { int rc_ = [&]() -> int { CK(call); return CLIFFS_OK; }(); if (rc_) return fail(rc_); } while (0)
+    const long long fs = (long long)g->B * g->plane;
     for (int k = 0; k < 2; ++k) {
-        CKG(cudaMalloc(&g->eta[k], sb)); CKG(cudaMalloc(&g->u[k], sb)); CKG(cudaMalloc(&g->v[k], sb));
-        CKG(cudaMemsetAsync(g->eta[k], 0, sb, g->stream));
-        CKG(cudaMemsetAsync(g->u[k], 0, sb, g->stream));
-        CKG(cudaMemsetAsync(g->v[k], 0, sb, g->stream));
+        CKG(cudaMalloc(&g->st[k], 3 * sb));
+        CKG(cudaMemsetAsync(g->st[k], 0, 3 * sb, g->stream));
+        g->eta[k] = g->st[k];
+        g->u[k] = g->st[k] + fs;
+        g->v[k] = g->st[k] + 2 * fs;
     }
-    CKG(cudaMalloc(&g->emax, sb)); CKG(cudaMalloc(&g->smax, sb));
+    CKG(cudaMalloc(&g->emax, 2 * sb));
+    g->smax = g->emax + fs;
     CKG(cudaMalloc(&g->d32, sizeof(float) * g->plane));
     CKG(cudaMalloc(&g->d64, sizeof(double) * (size_t)nx * ny));
     CKG(cudaMalloc(&g->d64b, sizeof(double) * (size_t)nx * ny));
     CKG(cudaMalloc(&g->xa, sizeof(float) * nx)); CKG(cudaMalloc(&g->xb, sizeof(float) * nx));
     CKG(cudaMalloc(&g->xk, sizeof(float) * nx)); CKG(cudaMalloc(&g->xrow, sizeof(float) * (ny + 2 * MET_PAD)));
     CKG(cudaMalloc(&g->ymet, sizeof(float4) * (ny + 2 * MET_PAD)));
+    CKG(cudaMalloc(&g->ymp, sizeof(float4) * (ny + 2 * MET_PAD)));
     CKG(cudaMalloc(&g->err, sizeof(int) * 4));
     CKG(cudaMemsetAsync(g->err, 0, sizeof(int) * 4, g->stream));
     CKG(cudaMalloc(&g->ured, sizeof(unsigned) * 4));
@@ -935,7 +994,7 @@ int cliffs_set_bathy(cliffs_grid* g, const double* x, const double* y, const dou
         for (int c = 0; c < nx; ++c) {
             const double l = f * ((c > 0) ? hx[c] - hx[c - 1] : hx[1] - hx[0]);
             const double r = f * ((c < nx - 1) ? hx[c + 1] - hx[c] : hx[nx - 1] - hx[nx - 2]);
-            xa[c] = (float)(1.0 / l); xb[c] = (float)(1.0 / r); xk[c] = (float)(dt * dt / (l + r));
+            xa[c] = (float)(0.5 / l); xb[c] = (float)(0.5 / r); xk[c] = (float)(dt * dt / (l + r));
         }
         if (sph) for (int j = 0; j < ny; ++j) xrow[j] = (float)(1.0 / (R_SPHERE * std::cos(hy[j] * DEGR)));
     }
@@ -945,7 +1004,7 @@ int cliffs_set_bathy(cliffs_grid* g, const double* x, const double* y, const dou
             const double l = f * ((j > 0) ? hy[j] - hy[j - 1] : hy[1] - hy[0]);
             const double r = f * ((j < ny - 1) ? hy[j + 1] - hy[j] : hy[ny - 1] - hy[ny - 2]);
             const double src = sph ? dt * std::tan(hy[j] * DEGR) / R_SPHERE : 0.0;
-            ym[j] = make_float4((float)(1.0 / l), (float)(1.0 / r), (float)(dt * dt / (l + r)), (float)src);
+            ym[j] = make_float4((float)(0.5 / l), (float)(0.5 / r), (float)(dt * dt / (l + r)), (float)-src);
         }
     }
     CK(cudaMemcpyAsync(g->xa, xa.data(), sizeof(float) * nx, cudaMemcpyHostToDevice, s));
@@ -954,14 +1013,16 @@ int cliffs_set_bathy(cliffs_grid* g, const double* x, const double* y, const dou
     // row tables padded by MET_PAD rows on each side (edge rows repeated), so that the
     // kernels index them without clamping
     std::vector<float> xrow_p(ny + 2 * MET_PAD);
-    std::vector<float4> ym_p(ny + 2 * MET_PAD);
+    std::vector<float4> ym_p(ny + 2 * MET_PAD), ymp_p(ny + 2 * MET_PAD);
     for (int j = 0; j < ny + 2 * MET_PAD; ++j) {
         const int jj = std::min(std::max(j - MET_PAD, 0), ny - 1);
         xrow_p[j] = xrow[jj];
         ym_p[j] = ym[jj];
+        ymp_p[j] = make_float4(ym[jj].y, ym[jj].y, ym[jj].z, ym[jj].z);
     }
     CK(cudaMemcpyAsync(g->xrow, xrow_p.data(), sizeof(float) * xrow_p.size(), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(g->ymet, ym_p.data(), sizeof(float4) * ym_p.size(), cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(g->ymp, ymp_p.data(), sizeof(float4) * ymp_p.size(), cudaMemcpyHostToDevice, s));
     CK(cudaStreamSynchronize(s));
     k_depth_to_f32<<<nblk((long long)ny * g->pitch), 256, 0, s>>>(g->d64, g->d32, nx, ny, g->pitch);
     CK(cudaGetLastError());
@@ -1033,19 +1094,34 @@ int cliffs_set_bathy(cliffs_grid* g, const double* x, const double* y, const dou
         CK(cudaMemcpy(g->items_d, g->samples.data(), sizeof(int4) * g->samples.size(), cudaMemcpyHostToDevice));
     }
     if (nx >= 3 && ny >= 3) {
-        // strips whose 64-column window holds a node that is dry at rest (d < h_min), or
-        // reaches the domain edge
-        std::vector<double> hd((size_t)nx * ny);
-        CK(cudaMemcpy(hd.data(), g->d64, sizeof(double) * hd.size(), cudaMemcpyDeviceToHost));
         const int nstrips = fused_strips(nx);
-        g->hard.assign(nstrips, 0);
-        for (int st = 0; st < nstrips; ++st) {
-            const int c0 = st * XOUT, c1 = c0 + XWIN;
-            if (c0 == 0 || c1 >= nx) { g->hard[st] = 1; continue; }
-            for (int j = 0; j < ny && !g->hard[st]; ++j)
-                for (int c = c0; c < c1; ++c)
-                    if (hd[(size_t)j * nx + c] < g->cfg.h_min) { g->hard[st] = 1; break; }
+        const size_t nh = (size_t)nstrips * ny;
+        int rct = ensure_tmp(g, nh);
+        if (rct) return rct;
+        CK(cudaMemsetAsync(g->tmp, 0, nh, s));
+        k_hard_rows<<<nblk((long long)nh, 8), 256, 0, s>>>(g->d32, nx, ny, g->pitch, nstrips, (float)g->cfg.h_min,
+                                                          g->cfg.itopo ? -3.402823466e38f : (float)g->cfg.dwall,
+                                                          (unsigned char*)g->tmp);
+        CK(cudaGetLastError());
+        g->hard.resize(nh);
+        CK(cudaMemcpyAsync(g->hard.data(), g->tmp, nh, cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        for (int st = 0; st < nstrips; ++st) {           // widened by three rows each way
+            unsigned char* h = g->hard.data() + (size_t)st * ny;
+            int last = -4;
+            for (int r = 0; r < ny; ++r) {
+                if (h[r] == 1) last = r;
+                else if (r - last <= 3) h[r] = 2;
+            }
+            last = ny + 3;
+            for (int r = ny - 1; r >= 0; --r) {
+                if (h[r] == 1) last = r;
+                else if (last - r <= 3) h[r] = 2;
+            }
         }
+        g->strip_cost.assign(nstrips, 0.0);
+        for (int st = 0; st < nstrips; ++st)
+            for (int r = 0; r < ny; ++r) g->strip_cost[st] += strip_row_cost(g, st, r);
     }
     int rc = choose_geometry(g);
     if (rc) return rc;
@@ -1296,7 +1372,8 @@ int cliffs_step_n(cliffs_grid* g, int64_t n) {
         fill_step_args(g, a, in, out);
         a.step = st;
         a.yfirst = g->cfg.alternate && ((st - 1) & 1);       // odd steps sweep y first
-        if (st % g->cfg.maxout == 0) { a.emax = g->emax; a.smax = g->smax; }
+        if (st % g->cfg.maxout == 0) a.emax = g->emax;
+        fused_ring(a.emax != nullptr, &a.nslots, &a.slot_floats);
         if (g->G && st % g->cfg.gout == 0) a.rec_g = g->grec + (st / g->cfg.gout) * g->G * 3;
         if (g->NN && st % g->cfg.bndout == 0) a.rec_n = g->nrec + (st / g->cfg.bndout) * g->NN * 3;
         if (g->inject_cycles > 0) {
@@ -1372,7 +1449,8 @@ int cliffs_run_persistent(cliffs_grid* g, int64_t n) {
     struct Key { StepArgs a; BatchArgs b; } k;
     std::memset(&k, 0, sizeof(k));
     fill_step_args(g, k.a, 0, 1);
-    k.a.eta_out = k.a.u_out = k.a.v_out = nullptr;
+    k.a.eta_out = nullptr;
+    fused_ring(last >= g->cfg.maxout, &k.a.nslots, &k.a.slot_floats);
     k.a.eta_in = k.a.u_in = k.a.v_in = nullptr;
     k.a.limit = nullptr;
     if (g->inject_cycles > 0) {
@@ -1387,8 +1465,8 @@ int cliffs_run_persistent(cliffs_grid* g, int64_t n) {
     b.nact = g->nact_d;
     b.nact_len = g->nact_len;
     b.nall = g->B;
-    for (int i = 0; i < 2; ++i) { b.eta[i] = g->eta[i]; b.u[i] = g->u[i]; b.v[i] = g->v[i]; }
-    b.emax = g->emax; b.smax = g->smax;
+    for (int i = 0; i < 2; ++i) b.eta[i] = g->eta[i];
+    b.emax = g->emax;
     b.maxout = g->cfg.maxout; b.gout = g->cfg.gout; b.bndout = g->cfg.bndout;
     b.grec = g->G ? g->grec : nullptr;
     b.grec_row = (long long)g->G * 3;
@@ -1558,8 +1636,8 @@ static int adjoint_yfirst_step(cliffs_grid* g, const StepArgs& a, const AdjLineA
         le = launch_transpose(LT + f * TPL, tp, LB + f * P, g->pitch, nx, ny, s);
     StepArgs ay = a;                                             // y-sweep of X_j
     ay.eta_in = st; ay.u_in = st + fst; ay.v_in = st + 2 * fst;
-    ay.eta_out = XR; ay.u_out = XR + P; ay.v_out = XR + 2 * P;
-    ay.emax = ay.smax = nullptr; ay.rec_g = ay.rec_n = nullptr; ay.samp_ptr = nullptr; ay.limit = nullptr;
+    ay.eta_out = XR; ay.fs_out = P;
+    ay.emax = nullptr; ay.rec_g = ay.rec_n = nullptr; ay.samp_ptr = nullptr; ay.limit = nullptr;
     ay.nstrips = (nx + XWIN - 1) / XWIN; ay.S = 64; ay.nseg = (ny + 63) / 64;
     if (le == cudaSuccess) le = launch_ysweep(ay, 1, s);
     AdjLineArgs X2 = X;                                          // x-sweep adjoint over it
@@ -1639,9 +1717,7 @@ static int adjoint_core(cliffs_grid* g, int scenario, int64_t n, int32_t checkpo
             StepMaps& M = g->adj_maps[j];
             M = g->maps[0];
             float* b = g->adj_slots + 3 * P * (size_t)NG * j;
-            int rc = make_map(&M.e, b, 3, g->pitch, ny, NG);
-            if (!rc) rc = make_map(&M.u, b + (size_t)NG * P, 3, g->pitch, ny, NG);
-            if (!rc) rc = make_map(&M.v, b + (size_t)2 * NG * P, 3, g->pitch, ny, NG);
+            const int rc = make_map(&M.s, b, g->pitch, ny, NG, (long long)NG * P, 3);
             if (rc) return rc;
         }
     }
@@ -1652,20 +1728,9 @@ static int adjoint_core(cliffs_grid* g, int scenario, int64_t n, int32_t checkpo
     if (NG > 1) {
         const long long cap = resident_warps(g) * ADJ_GROUP_WAVES;
         int Sr = 16;
-        for (; Sr < ny; Sr += 2) {
-            long long nw = 0;
-            for (int st = 0; st < g->nstrips; ++st) {
-                const int seg = (!g->hard.empty() && g->hard[st]) ? hard_rows(Sr) : Sr;
-                nw += (ny + seg - 1) / seg;
-            }
-            if (nw * NG <= cap) break;
-        }
+        while (Sr < ny && fused_warps(g, Sr) / g->B * NG > cap) Sr += 2;
         if (Sr != g->adj_S || g->adj_items.empty()) {
-            g->adj_items.clear();
-            for (int st = 0; st < g->nstrips; ++st) {
-                const int seg = (!g->hard.empty() && g->hard[st]) ? hard_rows(Sr) : Sr;
-                for (int r0 = 0; r0 < ny; r0 += seg) g->adj_items.push_back(make_int4(st, r0, std::min(r0 + seg, ny), 0));
-            }
+            cut_items(g, Sr, g->adj_items);
             cudaFree(g->adj_items_dev);
             g->adj_items_dev = nullptr;
             CK(cudaMalloc(&g->adj_items_dev, sizeof(int4) * g->adj_items.size()));
@@ -1721,7 +1786,7 @@ static int adjoint_core(cliffs_grid* g, int scenario, int64_t n, int32_t checkpo
     // (fields fout apart)
     auto step1 = [&](float* in, long long fin, const StepMaps& M, float* out, long long fout, long long j) -> int {
         a.eta_in = in; a.u_in = in + fin; a.v_in = in + 2 * fin;
-        a.eta_out = out; a.u_out = out + fout; a.v_out = out + 2 * fout;
+        a.eta_out = out; a.fs_out = fout;
         a.yfirst = g->cfg.alternate && ((s0 + j) & 1);     // the forward's parity: steps since set_initial
         a.items = g->items_dev;
         a.nitems = (int)g->items.size();
@@ -1738,7 +1803,7 @@ static int adjoint_core(cliffs_grid* g, int scenario, int64_t n, int32_t checkpo
     auto fwd = [&](int from, int to, long long j, int nb) -> int {
         if (nb == 1) return step1(slot(from), FS, g->adj_maps[from], slot(to), FS, j);
         a.eta_in = slot(from); a.u_in = slot(from) + FS; a.v_in = slot(from) + 2 * FS;
-        a.eta_out = slot(to); a.u_out = slot(to) + FS; a.v_out = slot(to) + 2 * FS;
+        a.eta_out = slot(to); a.fs_out = FS;
         a.yfirst = 0;
         a.items = g->adj_items_dev;
         a.nitems = (int)g->adj_items.size();
@@ -1794,9 +1859,7 @@ static int adjoint_core(cliffs_grid* g, int scenario, int64_t n, int32_t checkpo
                 StepMaps& M = g->adj_ppmaps[k];
                 M = g->maps[0];
                 float* b = g->adj_pp + 3 * P * k;
-                int rc = make_map(&M.e, b, 3, g->pitch, ny, 1);
-                if (!rc) rc = make_map(&M.u, b + P, 3, g->pitch, ny, 1);
-                if (!rc) rc = make_map(&M.v, b + 2 * P, 3, g->pitch, ny, 1);
+                const int rc = make_map(&M.s, b, g->pitch, ny, 1, P, 3);
                 if (rc) return rc;
             }
         }
@@ -1812,9 +1875,7 @@ static int adjoint_core(cliffs_grid* g, int scenario, int64_t n, int32_t checkpo
                 StepMaps& Mq = g->adj_pmaps[q];
                 Mq = g->maps[0];
                 float* b = at(j);
-                int rc = make_map(&Mq.e, b, 3, g->pitch, ny, 1);
-                if (!rc) rc = make_map(&Mq.u, b + FS, 3, g->pitch, ny, 1);
-                if (!rc) rc = make_map(&Mq.v, b + 2 * FS, 3, g->pitch, ny, 1);
+                const int rc = make_map(&Mq.s, b, g->pitch, ny, 1, FS, 3);
                 if (rc) return rc;
                 g->adj_pmaps_ok[q] = 1;
             }
@@ -1859,9 +1920,7 @@ static int adjoint_core(cliffs_grid* g, int scenario, int64_t n, int32_t checkpo
     X.xa = a.xa; X.xb = a.xb; X.xk = a.xk; X.xrow = a.xrow;
     X.gxy = g->adj_gxy; X.G = G;
     for (AdjLineArgs* A : {&X, &Y}) {
-        A->hmin = a.hmin; A->dwall = a.dwall; A->half_dt = a.half_dt; A->dt_gn2 = a.dt_gn2;
-        A->transverse = a.transverse;
-        A->inv_dt2_s1 = a.inv_dt2_s1;
+        A->K = a.K;
     }
     X.open_lo = g->cfg.open_edges & 1; X.open_hi = (g->cfg.open_edges >> 1) & 1;     // W, E
     Y.open_lo = (g->cfg.open_edges >> 2) & 1; Y.open_hi = (g->cfg.open_edges >> 3) & 1;   // S, N
@@ -1977,7 +2036,7 @@ int cliffs_set_rows_per_warp(cliffs_grid* g, int32_t rows) {
     if (!g->have_bathy) return set_err(CLIFFS_ERR_STATE, "set_bathy first (it chooses the geometry)");
     if (g->kind != 0) return set_err(CLIFFS_ERR_ARG, "a 1D grid has no tile shape");
     if (rows < 1 || rows > 8192) return set_err(CLIFFS_ERR_ARG, "rows per warp %d outside 1..8192", rows);
-    return set_rows_per_warp(g, rows, hard_rows(rows));
+    return set_rows_per_warp(g, rows);
 }
 
 int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32_t* ncand) {
@@ -2002,11 +2061,9 @@ int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32
     StepArgs a;
     fill_step_args(g, a, cur, 1 - cur);
     a.eta_out = scratch;
-    a.u_out = scratch + (size_t)g->B * g->plane;
-    a.v_out = scratch + 2 * (size_t)g->B * g->plane;
     a.step = g->step + 1;
     // fixed shapes, and those that just fit one, two or three waves of resident warps
-    std::vector<int> list = {16, 24, 32, 48, 64, 96, 128};
+    std::vector<int> list = {8, 16, 24, 32, 48, 64, 96, 128};
     for (int wv = 1; wv <= 3; ++wv) {
         const int S1 = wave_rows(g, wv);
         if (S1 > 0)
@@ -2024,7 +2081,7 @@ int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32
     int rc = CLIFFS_OK;
     for (int S : list) {
         if (S > 2 * g->ny && S != list[0]) break;
-        rc = set_rows_per_warp(g, S, hard_rows(S));
+        rc = set_rows_per_warp(g, S);
         if (rc) break;
         a.S = g->S; a.nseg = g->nseg; a.samp_ptr = g->samp_ptr; a.samp = g->samp;
         a.items = g->items_dev; a.nitems = (int)g->items.size();
@@ -2052,7 +2109,7 @@ int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32
     int h[4] = {0, 0, 0, 0};
     cudaMemcpy(h, g->err, sizeof(h), cudaMemcpyDeviceToHost);
     cudaMemset(g->err, 0, sizeof(h));
-    const int rc2 = set_rows_per_warp(g, rc ? oldS : bestS, hard_rows(rc ? oldS : bestS));
+    const int rc2 = set_rows_per_warp(g, rc ? oldS : bestS);
     if (ncand) *ncand = n;
     if (rc) return rc;
     if (rc2) return rc2;

@@ -1,15 +1,14 @@
 // Sweep kernels of the split shallow-water step (arXiv 1410.0753, section "Numerics").
 //
 //  k_step_fused  one full step (x-sweep then y-sweep) per launch. A warp owns a strip of
-//                56 output columns and S output rows. It walks the rows of its strip from
-//                r0-3 to r0+S+2. Each row (64 columns of eta, u, v, d and, when max-wave is
-//                due, the max-wave rows three rows behind) arrives in shared memory by TMA
-//                (cp.async.bulk.tensor) through a 4-slot ring per warp with one mbarrier per
-//                slot; one lane keeps the ring RING rows ahead. The row is x-swept across the
-//                warp with shuffles and pushed into a per-column register pipeline that
-//                finishes the y-sweep three rows behind. The step reads eta, u, v, d and
-//                writes eta, u, v once per cell (28 B/cell-update plus the halo), fused with
-//                the max-wave update (+8 B) and the gauge / enclosed-grid sampling.
+//                56 output columns and S output rows. The rows of its strip arrive in shared
+//                memory by TMA (cp.async.bulk.tensor: one box of eta, u, v and one of d per
+//                four rows) through a ring per warp with one mbarrier per slot. Each row
+//                (64 columns) is x-swept across the warp with shuffles and enters a
+//                per-column register march that finishes the y-sweep two or three rows
+//                behind. The step reads eta, u, v, d and writes eta, u, v once per cell
+//                (28 B/cell-update plus the halo), fused with the max-wave update (+8 B) and
+//                the gauge / enclosed-grid sampling.
 //  k_batch       the same per-warp work in a persistent cooperative kernel that loops over
 //                the steps of a batch of scenarios, with a grid barrier between steps.
 //  k_xsweep      x-sweep alone (1D grids along x).
@@ -25,7 +24,6 @@
 namespace cliffs {
 
 // ------------------------------------------------------------------ launchers
-// the ring needs more than the default 48 KB of dynamic shared memory per block
 // Kernel variants, indexed by the grid's metric (spherical: +1), friction (on: +2), sweep
 // order of the step (y first: +4) and solver (eq. (solver1): +8 for the fused step, +4 for
 // the others); grids with open outer edges take the OPEN instantiations of the same tables.
@@ -62,8 +60,19 @@ static const void* ysweep_kernel(bool sph, bool fric, bool s1, bool open) {
     return open ? ysweep_kernel_open(v) : t[v];
 }
 
-static bool solver1(const StepArgs& a) { return a.inv_dt2_s1 > 0.f; }
+static bool solver1(const StepArgs& a) { return a.K.inv_dt2 > 0.f; }
 
+// Dynamic shared memory of a block: the mbarriers and the warps' rings.
+static int fused_smem(int nslots, int slot_floats) { return BAR_BYTES + FUSED_WARPS * nslots * slot_floats * 4; }
+// The ring without max-wave rows: three slots of eta, u, v, d (12 KB per warp); with them two
+// slots of six arrays, the same size.
+void fused_ring(bool maxwave, int* nslots, int* slot_floats) {
+    *nslots = maxwave ? 2 : 3;
+    *slot_floats = (maxwave ? 6 : 4) * ARR_FLOATS;
+}
+static const int FUSED_SMEM = fused_smem(3, 4 * ARR_FLOATS);
+
+// the ring needs more than the default 48 KB of dynamic shared memory per block
 static cudaError_t fused_smem_optin() {
     static cudaError_t done = cudaErrorNotReady;
     if (done == cudaErrorNotReady) {
@@ -85,8 +94,8 @@ cudaError_t launch_step_fused(const StepArgs& a, const StepMaps& m, int batch, c
     StepMaps mm = m;
     StepArgs aa = a;
     void* args[] = {&mm, &aa};
-    return cudaLaunchKernel(fused_kernel(a.sph, a.dt_gn2 > 0.f, a.yfirst != 0, solver1(a), a.open_edges != 0), grid,
-                            dim3(FUSED_WARPS * 32), args, FUSED_SMEM, s);
+    return cudaLaunchKernel(fused_kernel(a.sph, a.K.fric != 0, a.yfirst != 0, solver1(a), a.open_edges != 0), grid,
+                            dim3(FUSED_WARPS * 32), args, fused_smem(a.nslots, a.slot_floats), s);
 }
 
 cudaError_t launch_batch(const StepArgs& a, const StepMaps2& mm, const BatchArgs& b, int blocks, cudaStream_t s) {
@@ -95,7 +104,7 @@ cudaError_t launch_batch(const StepArgs& a, const StepMaps2& mm, const BatchArgs
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(FUSED_WARPS * 32);
-    cfg.dynamicSmemBytes = FUSED_SMEM;
+    cfg.dynamicSmemBytes = fused_smem(a.nslots, a.slot_floats);
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeCooperative;         // all blocks resident: the grid barrier
@@ -106,7 +115,7 @@ cudaError_t launch_batch(const StepArgs& a, const StepMaps2& mm, const BatchArgs
     StepArgs aa = a;
     BatchArgs bb = b;
     void* args[] = {&m2, &aa, &bb};
-    return cudaLaunchKernelExC(&cfg, batch_kernel(a.sph, a.dt_gn2 > 0.f, solver1(a), a.open_edges != 0, b.alternate != 0), args);
+    return cudaLaunchKernelExC(&cfg, batch_kernel(a.sph, a.K.fric != 0, solver1(a), a.open_edges != 0, b.alternate != 0), args);
 }
 
 int batch_blocks_per_sm(bool sph) {
@@ -130,7 +139,7 @@ cudaError_t launch_xsweep(const StepArgs& a, int batch, cudaStream_t s) {
     const dim3 grid((a.nstrips * a.ny + 3) / 4, batch);
     StepArgs aa = a;
     void* args[] = {&aa};
-    return cudaLaunchKernel(xsweep_kernel(a.sph, a.dt_gn2 > 0.f, solver1(a), a.open_edges != 0), grid, dim3(128), args, 0, s);
+    return cudaLaunchKernel(xsweep_kernel(a.sph, a.K.fric != 0, solver1(a), a.open_edges != 0), grid, dim3(128), args, 0, s);
 }
 
 cudaError_t launch_ysweep(const StepArgs& a, int batch, cudaStream_t s) {
@@ -138,7 +147,7 @@ cudaError_t launch_ysweep(const StepArgs& a, int batch, cudaStream_t s) {
     const dim3 grid((nw + 3) / 4, batch);
     StepArgs aa = a;
     void* args[] = {&aa};
-    return cudaLaunchKernel(ysweep_kernel(a.sph, a.dt_gn2 > 0.f, solver1(a), a.open_edges != 0), grid, dim3(128), args, 0, s);
+    return cudaLaunchKernel(ysweep_kernel(a.sph, a.K.fric != 0, solver1(a), a.open_edges != 0), grid, dim3(128), args, 0, s);
 }
 
 }  // namespace cliffs

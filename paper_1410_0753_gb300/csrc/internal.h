@@ -7,17 +7,34 @@
 
 namespace cliffs {
 
+// Constants of a sweep. Those that enter packed FP32x2 arithmetic are kept as pairs, so that
+// no instruction is spent on widening them.
+struct SweepConst {
+    float hmin;       // h_min ('ground')
+    float dwall;      // nodes with d < dwall are permanent walls (-FLT_MAX when itopo != 0)
+    float half_dt;    // dt / 2
+    float inv_dt2;    // 1 / dt^2 with eq. (solver1) (1/(dx_{j-1}+dx_j) = k2 / dt^2), else 0
+    int fric;         // friction on
+    int transverse;   // eq. (pq3) on/off
+    float2 hdt;       // dt / 2
+    float2 ntr;       // -1 with eq. (pq3), 0 without
+    float2 lgf;       // log2(dt g n^2 g^(4/3)) (friction, fric_k2)
+};
+
 // Arguments of one sweep-kernel launch (all device pointers). Fields 2D are pitched:
 // element (b, r, c) lives at b * plane + r * pitch + c.
 struct StepArgs {
     const float* eta_in; const float* u_in; const float* v_in;
-    float* eta_out; float* u_out; float* v_out;
+    float* eta_out;                  // u and v follow at the field stride
+    long long fs_out;                // floats from eta to u and from u to v of the output state
     const float* d;                  // [ny][pitch], FP32 depth
-    const float* xa; const float* xb; const float* xk;   // [nx] per-column x metric
+    const float* xa; const float* xb; const float* xk;   // [nx] per-column x metric: 1/(2 dx_{j-1}), 1/(2 dx_j), dt^2/(dx_{j-1}+dx_j)
     // per-row tables, valid for row indices -MET_PAD .. ny + MET_PAD - 1 (edge rows repeated)
     const float* xrow;               // row factor of the x metric (1 or 1/(R cos phi))
-    const float4* ymet;              // (1/dy_{j-1}, 1/dy_j, dt^2/(dy_{j-1}+dy_j), dt tan(phi)/R)
-    float* emax; float* smax;        // max-wave fields, or null when not due this step
+    const float4* ymet;              // (1/(2 dy_{j-1}), 1/(2 dy_j), dt^2/(dy_{j-1}+dy_j), -dt tan(phi)/R)
+    float* emax;                     // max-wave eta, or null when not due this step
+    long long fs_max;                // floats from the max-wave eta to the max-wave speed
+    const float4* ymp;               // (1/(2 dy_j) twice, dt^2/(dy_{j-1}+dy_j) twice): packed operands
     float* rec_g;                    // gauge record row of this step (scenario 0) or null
     float* rec_n;                    // enclosed-grid node record row or null
     long long rec_g_bstride;         // floats between scenarios in the gauge records
@@ -32,11 +49,11 @@ struct StepArgs {
     int nstrips, nseg;
     const int4* items;               // fused kernel: per warp (strip, first row, end row)
     int nitems;
-    float hmin, dwall, half_dt, dt_gn2;
-    int transverse;
+    int nslots, slot_floats;         // ring of a fused warp: slots and floats per slot
+    int walls;                       // itopo = 0: nodes with d < dwall are walls
+    SweepConst K;
     int sph;                         // geographic grid: x metric scaled per row
     int yfirst;                      // this step sweeps y, then x (alternating order)
-    float inv_dt2_s1;                // 1/dt^2 with eq. (solver1), 0 with eq. (solver2)
     int open_edges;                  // open outer edges: bits W 1, E 2, S 4, N 8
     long long wait_cycles;           // limit of every mbarrier wait (clock cycles)
     unsigned tx_pad;                 // extra bytes each ring slot expects (fault injection; 0)
@@ -45,7 +62,7 @@ struct StepArgs {
 enum { ERRF_NONFINITE = 1, ERRF_TIMEOUT = 2 };
 constexpr int MET_PAD = 8;
 constexpr int TMA_BOX_COLS = 64;   // columns of one TMA box (a warp's window)
-constexpr int TMA_BOX_ROWS = 2;    // rows of one TMA box (one ring slot)
+constexpr int TMA_BOX_ROWS = 4;    // rows of one TMA box (one ring slot)
 
 // Depth-jump filter (section "Numerical stability", eqs. (dstab), (newdw), (newdc)), one
 // node per thread; shared by cliffs_set_bathy and cliffs_depth_filter_noalloc so that both
@@ -84,10 +101,11 @@ __device__ __forceinline__ void filter_pass_node(const double* in, double* out, 
 // message returned by cliffs_last_error() on the calling thread (cliffs_api.cu)
 void set_last_error(const char* msg);
 
-// TMA descriptors of the fused step's inputs: eta, u, v, eta_max, speed_max as 3D
-// [batch][ny][pitch] tensors and d as a 2D [ny][pitch] tensor, each read as 64 x 1 boxes.
+// TMA descriptors of the fused step's inputs: the state as a 4D [3][batch][ny][pitch] tensor
+// (eta, u, v), d as a 2D [ny][pitch] tensor and the max-wave fields as [2][batch][ny][pitch],
+// each read as 64 x 4 boxes, every field of the state (of the maxima) in one box.
 struct StepMaps {
-    CUtensorMap e, u, v, d, em, sm;
+    CUtensorMap s, d, mw;
 };
 
 struct StepMaps2 {
@@ -110,8 +128,8 @@ struct BatchArgs {
     const int* nact;                 // [nact_len]: scenarios whose limit is >= the step; null: all
     long long nact_len;
     int nall;                        // the batch size
-    float* eta[2]; float* u[2]; float* v[2];
-    float* emax; float* smax;
+    float* eta[2];                   // u and v at the field stride (StepArgs.fs_out)
+    float* emax;
     int maxout, gout, bndout;
     float* grec;                     // gauge records, row = step / gout (scenario stride in StepArgs)
     long long grec_row;              // floats per record row
@@ -154,6 +172,7 @@ cudaError_t launch_batch(const StepArgs& a, const StepMaps2& mm, const BatchArgs
 int batch_blocks_per_sm(bool sph);
 cudaError_t launch_step_fused(const StepArgs& a, const StepMaps& m, int batch, cudaStream_t s);
 int fused_blocks_per_sm(bool sph);
+void fused_ring(bool maxwave, int* nslots, int* slot_floats);
 int fused_warps_per_block();
 cudaError_t launch_xsweep(const StepArgs& a, int batch, cudaStream_t s);
 cudaError_t launch_ysweep(const StepArgs& a, int batch, cudaStream_t s);

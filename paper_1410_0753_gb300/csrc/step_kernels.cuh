@@ -7,15 +7,12 @@
 
 namespace cliffs {
 
-constexpr int RING = 4;                       // slots in flight per warp
-constexpr int SLOT_ROWS = TMA_BOX_ROWS;       // rows per slot (one TMA box each array)
-static_assert(TMA_BOX_COLS == XWIN, "a TMA box spans the warp's window");
-constexpr int NARR = 6;                       // eta, u, v, d, eta_max, speed_max
-constexpr int ARR_FLOATS = SLOT_ROWS * XWIN;
-constexpr int SLOT_FLOATS = NARR * ARR_FLOATS;
-constexpr int WARP_RING_BYTES = RING * SLOT_FLOATS * 4;
+constexpr int SLOT_ROWS = TMA_BOX_ROWS;       // rows per ring slot (one TMA box per tensor)
+static_assert(TMA_BOX_COLS == XWIN && SLOT_ROWS == 4, "a TMA box spans the warp's window");
+constexpr int ARR_FLOATS = SLOT_ROWS * XWIN;  // one array of a slot: eta, u, v, d [, eta_max, speed_max]
 constexpr int FUSED_WARPS = 4;
-constexpr int FUSED_SMEM = FUSED_WARPS * (WARP_RING_BYTES + RING * 8);
+constexpr int MAX_SLOTS = 8;                  // mbarriers kept per warp
+constexpr int BAR_BYTES = FUSED_WARPS * MAX_SLOTS * 8;
 
 // ------------------------------------------------------------------ TMA / mbarrier (PTX)
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
@@ -50,13 +47,25 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, unsigned parity, long lon
         if (clock64() - t0 > limit) return false;
     return true;
 }
-__device__ __forceinline__ void tma_row3(float* dst, const CUtensorMap* m, uint64_t* b, int x, int y, int z) {
+__device__ __forceinline__ void tma_box4(float* dst, const CUtensorMap* m, uint64_t* b, int x, int y, int z) {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(b)), "r"(x), "r"(y), "r"(z)
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4, %5, %6}], [%2];"
+        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(b)), "r"(x), "r"(y), "r"(z), "r"(0)
         : "memory");
 }
+__device__ __forceinline__ void tma_box2(float* dst, const CUtensorMap* m, uint64_t* b, int x, int y) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4}], [%2];"
+        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(b)), "r"(x), "r"(y)
+        : "memory");
+}
+
+// A value that is the same in every lane, through an instruction whose result is uniform by
+// construction: the compiler then keeps what derives from it (row counters, ring positions)
+// in uniform registers and branches on it without convergence barriers.
+__device__ __forceinline__ int uniform(int x) { return __reduce_max_sync(FULL, x); }
 
 // ------------------------------------------------------------------ epilogue
 // Nodes (r, c) and (r, c+1) of the step input, for the kernels without TMA; nodes outside
@@ -97,339 +106,485 @@ __device__ __forceinline__ int runaway(float e, float u, float v) {
 constexpr float RUNAWAY_SQ = 9e10f;
 
 // What changes from one step to the next: the input state's TMA descriptors, the output
-// planes, and the max-wave fields and record rows when they are due this step (else null).
+// planes (eta; u and v follow at the field stride), and the max-wave fields and record rows
+// when they are due this step (else null).
 struct StepOut {
     const StepMaps* M;
     float* eta_out;
-    float* u_out;
-    float* v_out;
     float* emax;
-    float* smax;
     float* rec_g;
     float* rec_n;
 };
 
 __device__ __forceinline__ StepOut step_out(const StepMaps* M, const StepArgs& a) {
-    return StepOut{M, a.eta_out, a.u_out, a.v_out, a.emax, a.smax, a.rec_g, a.rec_n};
+    return StepOut{M, a.eta_out, a.emax, a.rec_g, a.rec_n};
 }
 
-// Store a finished pair of nodes of row r. With max-wave due (section "Running Options",
-// field maxout), (em, sm) hold the stored maxima of the pair (loaded beforehand); on wet
-// nodes they take the new eta and speed sqrt(u^2 + v^2) where these are larger and are
-// written back.
-// With CHECK the runaway test runs here (the fused kernels accumulate it instead, chk_out).
-template <bool CHECK = true>
-__device__ __forceinline__ void emit_pair(const StepArgs& a, const StepOut& O, size_t o, bool va, bool vb,
-                                          float2 E, float2 U, float2 V, float2 D,
-                                          float2 em, float2 sm, int& bad) {
-    if (!va) return;
+// Store a finished pair of nodes at po (eta; u and v at the field stride fs). With max-wave
+// due (section "Running Options", field maxout), (em, sm) hold the stored maxima of the pair
+// and pm is where they live (speed at the stride ms): on wet nodes they take the new eta and
+// speed sqrt(u^2 + v^2) where these are larger and are written back.
+__device__ __forceinline__ void emit_pair(float* po, long long fs, bool va, bool vb,
+                                          float2 E, float2 U, float2 V) {
     if (vb) {
-        *reinterpret_cast<float2*>(O.eta_out + o) = E;
-        *reinterpret_cast<float2*>(O.u_out + o) = U;
-        *reinterpret_cast<float2*>(O.v_out + o) = V;
-        if (CHECK) bad |= runaway(E.x, U.x, V.x) | runaway(E.y, U.y, V.y);
-    } else {
-        O.eta_out[o] = E.x; O.u_out[o] = U.x; O.v_out[o] = V.x;
-        if (CHECK) bad |= runaway(E.x, U.x, V.x);
+        *reinterpret_cast<float2*>(po) = E;
+        *reinterpret_cast<float2*>(po + fs) = U;
+        *reinterpret_cast<float2*>(po + 2 * fs) = V;
+    } else if (va) {
+        po[0] = E.x; po[fs] = U.x; po[2 * fs] = V.x;
     }
-    if (O.emax) {
-        // max-wave of the pair (wet nodes only), the tests in packed form
-        const float2 h = add2(E, D);
-        const float2 s2 = fma2(U, U, mul2(V, V));
-        const float2 sm2 = mul2(sm, sm);
-        const bool wA = (D.x >= a.dwall) && (h.x >= a.hmin);
-        const bool wB = vb && (D.y >= a.dwall) && (h.y >= a.hmin);
-        const bool eA = wA && E.x > em.x, eB = wB && E.y > em.y;
-        const bool sA = wA && s2.x > sm2.x, sB = wB && s2.y > sm2.y;
-        if (eA || eB || sA || sB) {
-            if (eA) em.x = E.x;
-            if (eB) em.y = E.y;
-            if (sA) sm.x = fmaxf(sm.x, sqrt_pos(s2.x));
-            if (sB) sm.y = fmaxf(sm.y, sqrt_pos(s2.y));
-            if (vb) {
-                *reinterpret_cast<float2*>(O.emax + o) = em;
-                *reinterpret_cast<float2*>(O.smax + o) = sm;
-            } else {
-                O.emax[o] = em.x; O.smax[o] = sm.x;
-            }
+}
+__device__ __forceinline__ void emit_max(const SweepConst& K, float* pm, long long ms, bool va, bool vb,
+                                         float2 E, float2 U, float2 V, float2 D, float2 em, float2 sm) {
+    const float2 h = add2(E, D);
+    const float2 s2 = fma2(U, U, mul2(V, V));
+    const float2 sm2 = mul2(sm, sm);
+    const bool wA = va && (D.x >= K.dwall) && (h.x >= K.hmin);
+    const bool wB = vb && (D.y >= K.dwall) && (h.y >= K.hmin);
+    const bool eA = wA && E.x > em.x, eB = wB && E.y > em.y;
+    const bool sA = wA && s2.x > sm2.x, sB = wB && s2.y > sm2.y;
+    if (eA || eB || sA || sB) {
+        if (eA) em.x = E.x;
+        if (eB) em.y = E.y;
+        if (sA) sm.x = fmaxf(sm.x, sqrt_pos(s2.x));
+        if (sB) sm.y = fmaxf(sm.y, sqrt_pos(s2.y));
+        if (vb) {
+            *reinterpret_cast<float2*>(pm) = em;
+            *reinterpret_cast<float2*>(pm + ms) = sm;
+        } else {
+            pm[0] = em.x; pm[ms] = sm.x;
         }
     }
 }
 
-// Gauge / enclosed-grid node samples owned by this warp, sorted by row. The warp keeps 32
-// consecutive sample records in registers (lane l holds record base + l). For a row with
-// samples, every lane whose record belongs to that row fetches the node's values from the
-// lane that owns the node by shuffle and writes the record, so all samples of a row go out
-// together; `next` holds the row of the next sample so rows without samples cost a compare.
-// The writer is a separate (not inlined) function: it runs on the few rows with samples,
-// and kept out of the row loop it leaves the loop's code to the sweeps.
-struct Samples {
-    int sp, se, base, next;
-    int4 mine;
-
-    __device__ __forceinline__ void load(const int4* samp, int lane) {
-        base = sp;
-        mine = (sp + lane < se) ? __ldg(samp + sp + lane) : make_int4(0x7fffffff, 0, 0, 0);
+// The gauge / enclosed-grid records of a work item whose rows are all stored: every lane reads
+// nodes of the item's sample list back from the output (written by this warp, so a warp
+// barrier orders it; the lines are in L2) and writes their records. Sampling inside the row
+// loop instead, from registers, took a call there and 18 warp-instructions per row whether
+// the row has samples or not (147.7 against 164.0 us on a 4096^2 grid without any).
+__device__ __forceinline__ void write_samples(const StepArgs& a, const StepOut& O, int item, int b, int lane) {
+    if (!a.samp_ptr || !(O.rec_g || O.rec_n)) return;
+    const int sp = __ldg(a.samp_ptr + item), se = __ldg(a.samp_ptr + item + 1);
+    if (sp >= se) return;
+    __syncwarp();
+    const float* st = O.eta_out + (long long)b * a.plane;
+    float* rg = O.rec_g ? O.rec_g + (long long)b * a.rec_g_bstride : nullptr;
+    for (int i = sp + lane; i < se; i += 32) {
+        const int4 it = __ldg(a.samp + i);           // (row, col, class 0 gauge / 1 node, slot)
+        float* out = it.z == 0 ? rg : O.rec_n;
+        if (!out) continue;
+        const float* q = st + ((long long)it.x * a.pitch + it.y);
+        const float e = q[0], u = q[a.fs_out], v = q[2 * a.fs_out];
+        out[3 * it.w + 0] = e;
+        out[3 * it.w + 1] = u;
+        out[3 * it.w + 2] = v;
     }
-    __device__ __forceinline__ void init(const StepArgs& a, const StepOut& O, int gw, int lane) {
-        sp = se = base = 0;
-        next = 0x7fffffff;
-        mine = make_int4(0x7fffffff, 0, 0, 0);
-        if (a.samp_ptr && (O.rec_g || O.rec_n)) {
-            sp = a.samp_ptr[gw];
-            se = a.samp_ptr[gw + 1];
-            if (sp < se) {
-                load(a.samp, lane);
-                next = __shfl_sync(FULL, mine.x, 0);
-            }
-        }
-    }
-    __device__ __forceinline__ void emit(const StepArgs& a, const StepOut& O, int b, int r, int c0,
-                                         int lane, float2 E, float2 U, float2 V);
-};
-
-// the samples of row r (warp-collective); returns the updated sample cursor
-static __device__ __noinline__ Samples samples_write(Samples S, const int4* samp, float* rec_g, float* rec_n, int r,
-                                                     int c0, int lane, float2 E, float2 U, float2 V) {
-    while (true) {
-        const bool mineRow = lane >= S.sp - S.base && S.mine.x == r;
-        const int rel = S.mine.y - c0;
-        const int src = mineRow ? (rel >> 1) & 31 : lane;
-        const float ex = __shfl_sync(FULL, E.x, src), ey = __shfl_sync(FULL, E.y, src);
-        const float ux = __shfl_sync(FULL, U.x, src), uy = __shfl_sync(FULL, U.y, src);
-        const float vx = __shfl_sync(FULL, V.x, src), vy = __shfl_sync(FULL, V.y, src);
-        if (mineRow) {
-            const bool isB = rel & 1;
-            float* out = (S.mine.z == 0) ? rec_g : rec_n;
-            if (out) {
-                out[3 * S.mine.w + 0] = isB ? ey : ex;
-                out[3 * S.mine.w + 1] = isB ? uy : ux;
-                out[3 * S.mine.w + 2] = isB ? vy : vx;
-            }
-        }
-        S.sp += __popc(__ballot_sync(FULL, mineRow));
-        if (S.sp >= S.se) { S.next = 0x7fffffff; return S; }
-        if (S.sp - S.base < 32) {                  // the next record is cached: a later row
-            S.next = __shfl_sync(FULL, S.mine.x, S.sp - S.base);
-            return S;
-        }
-        S.load(samp, lane);                        // the row's records run past the cache
-        S.next = __shfl_sync(FULL, S.mine.x, 0);
-        if (S.next != r) return S;
-    }
-}
-
-__device__ __forceinline__ void Samples::emit(const StepArgs& a, const StepOut& O, int b, int r, int c0,
-                                              int lane, float2 E, float2 U, float2 V) {
-    if (r != next) return;
-    *this = samples_write(*this, a.samp, O.rec_g ? O.rec_g + (long long)b * a.rec_g_bstride : nullptr, O.rec_n,
-                          r, c0, lane, E, U, V);
 }
 
 // ------------------------------------------------------------------ fused step
 // One warp of the fused step. A work item is a strip and an output row range [r0, r1); the
-// warp walks rows r0-3 .. r1+2 as pairs, one pair per ring slot. The ring's slot and phase
-// follow a running pair count, so a warp may process any number of items in a row. With YF
-// (a y-first step of the alternating order) rows enter the y-sweep pipeline unswept and each
-// finished row is x-swept across the warp on its way out; the tile geometry is the same.
+// warp marches down the rows of its 64-column window, which arrive by TMA in slots of four
+// rows (one box for eta, u, v and one for d, issued by one lane) through a ring per warp.
+//
+// One vote per row decides its path: when the incoming row k and the x-swept rows before it
+// are wet, the row is open water and one straight block of code updates row k-2 in the y-sweep
+// (which needs rows k-3 .. k-1 only) and x-sweeps row k, two independent chains of arithmetic
+// side by side; else the general x-sweep and march step run (slow_row). In open water a row
+// depends on one row above and below only, so the march starts at row r0-1 and ends with row
+// r1+1 in place of r0-3 .. r1+2; should one of the first rows turn out not to be open water,
+// it starts over from r0-3 (nothing has been written by then, and the first slot, which
+// holds rows r0-3 .. r0, is still there). At the top and bottom of the domain the walls are
+// set in the fast path, and rows past the domain only keep the march going.
+//
+// The ring's position and phase bits live as long as the warp, so a warp may process any
+// number of items in a row. With YF (a y-first step of the alternating order) rows enter the
+// march unswept and each finished row is x-swept across the warp on its way out.
 template <bool SPH, bool FRIC, bool YF = false, bool S1 = false, bool OPEN = false>
 struct FusedWarp {
+    // the plain step has its open-water loop once per case (edge windows, max-wave due); the
+    // other variants one loop for all
+    static constexpr bool MAIN = !YF && !S1 && !OPEN;
     const StepArgs& a;
-    SweepConst K;
+    const SweepConst& K;
     float* ring;
     uint64_t* bar;
-    unsigned used;             // ring pairs consumed by this warp so far (2^32 is a multiple of 2 * RING)
-    int lane, b, c0, cA, r0, r1, k0, npairs;
-    size_t orow;               // output offset of row r0 (scenario plane + column)
-    bool colA, colB, vA, vB, edge;
-    bool bounded;              // the window starts or ends at the domain's edge (xsweep2)
-    unsigned tx, nbox;
-    unsigned ends;             // open outer edges among this lane's columns (open_ends_x)
-    XMet2 m0;
+    unsigned phase;            // phase parity of each ring slot (bits)
+    int head;                  // the ring slot to fill next
+    int cs;                    // the ring slot being read
+    int nfill, nread, ntot;    // slots of the item filled, waited for, to be filled
+    int lane, b, c0, r0, r1, k0, kpast;
+    bool sw;                   // this lane's nodes of row k-1 that count are wet at the start of the y-sweep
+    bool colA, colB, vA, vB;
+    bool wallx;                // the window touches the domain's edge
+    unsigned tx, ends, walls;
+    XMet2 m0;                  // hl is formed where it is needed
     YMarch2 ym;
-    Samples smp;
     StepOut O;
     int bad;
-    float2 chk_x;              // sum of 0 * (x-swept eta): 0, or NaN once a value is not finite
+    float2 chk_x;              // sum of 0 * (x-swept eta) of the general rows: 0, or NaN once one is not finite
     float2 chk_out;            // sum of e^2 + u^2 + v^2 over the stored nodes (RUNAWAY_SQ)
 
-    __device__ __forceinline__ FusedWarp(const StepArgs& a_) : a(a_) {}
-
+    __device__ __forceinline__ FusedWarp(const StepArgs& a_) : a(a_), K(a_.K) {}
     __device__ __forceinline__ void setup(unsigned char* smem_raw, int wib) {
         lane = threadIdx.x & 31;
-        K = SweepConst{a.hmin, a.dwall, a.half_dt, a.dt_gn2, a.transverse, a.inv_dt2_s1};
-        ring = reinterpret_cast<float*>(smem_raw + wib * WARP_RING_BYTES);
-        bar = reinterpret_cast<uint64_t*>(smem_raw + FUSED_WARPS * WARP_RING_BYTES) + wib * RING;
-        used = 0;
+        bar = reinterpret_cast<uint64_t*>(smem_raw) + wib * MAX_SLOTS;
+        ring = reinterpret_cast<float*>(smem_raw + BAR_BYTES) + wib * a.nslots * a.slot_floats + 2 * lane;
+        phase = 0u;
+        head = 0;
         bad = 0;
         chk_x = chk_out = v2(0.f);
         if (lane == 0) {
-            for (int s = 0; s < RING; ++s) mbar_init(&bar[s], 1);
+            for (int s = 0; s < a.nslots; ++s) mbar_init(&bar[s], 1);
             fence_mbar_init();
         }
         __syncwarp();
     }
 
-    // lanes 0..nbox-1 each start one 64 x 2 box of the item's row pair j into its ring slot
-    __device__ __forceinline__ void issue(int j) {
-        const int slot = (int)((used + (unsigned)j) % RING);
-        const int row = k0 + SLOT_ROWS * j;
-        if (lane == 0) mbar_arrive_tx(&bar[slot], tx);
-        if (lane < (int)nbox) {
-            fence_proxy_async();
-            tma_row3(ring + slot * SLOT_FLOATS + lane * ARR_FLOATS, &O.M->e + lane, &bar[slot], c0,
-                     lane >= 4 ? row - 3 : row, lane == 3 ? 0 : b);
+    __device__ __forceinline__ int next_of(int s) const { return s + 1 == a.nslots ? 0 : s + 1; }
+    // this lane's pair in row q of ring slot s
+    __device__ __forceinline__ const float* at(int s, int q) const { return ring + s * a.slot_floats + q * XWIN; }
+
+    // one lane starts the boxes of the item's next slot (rows k0 + 4 nfill ..; the max-wave
+    // rows two rows behind, where the open-water path emits)
+    __device__ __forceinline__ void fill() {
+        if (lane == 0) {
+            float* dst = ring + head * a.slot_floats;
+            const int row = k0 + SLOT_ROWS * nfill;
+            mbar_arrive_tx(&bar[head], tx);
+            tma_box4(dst, &O.M->s, &bar[head], c0, row, b);
+            tma_box2(dst + 3 * ARR_FLOATS, &O.M->d, &bar[head], c0, row);
+            if (O.emax) tma_box4(dst + 4 * ARR_FLOATS, &O.M->mw, &bar[head], c0, row - 2, b);
+        }
+        head = next_of(head);
+        ++nfill;
+    }
+    // wait for ring slot cs (bounded); false when it expired
+    __device__ __forceinline__ bool acquire() {
+        const bool ok = mbar_wait(&bar[cs], (phase >> cs) & 1u, a.wait_cycles);
+        if (!__all_sync(FULL, ok)) return false;
+        phase ^= 1u << cs;
+        ++nread;
+        return true;
+    }
+    // The march enters the slot that row k begins (`open`: the row only keeps open water going, so
+    // a row past the last slot is not read).
+    __device__ __forceinline__ bool next_slot(int k, bool open) {
+        cs = next_of(cs);
+        const int i = (k - k0) >> 2;
+        if (i < nread) return true;                     // started over: it is here already
+        if (i >= ntot && k < a.ny && !open) {           // rows past r1, for the general path
+            ntot = i + 1;
+            __syncwarp();
+            fill();
+        }
+        return i >= ntot || acquire();
+    }
+    // the slot before the one row k is in is free: its place takes a new one
+    __device__ __forceinline__ void refill(int k) {
+        if (nfill < ntot && nfill < ((k - k0) >> 2) + a.nslots) {
+            __syncwarp();
+            fill();
         }
     }
 
-    // row k held at `s`: its values (zero state, dry depth outside the domain) and x metric
-    __device__ __forceinline__ bool load_row(int k, const float* s, float2& E, float2& U, float2& V, float2& D,
-                                             XMet2& m) {
-        E = reinterpret_cast<const float2*>(s + 0 * ARR_FLOATS)[lane];
-        U = reinterpret_cast<const float2*>(s + 1 * ARR_FLOATS)[lane];
-        V = reinterpret_cast<const float2*>(s + 2 * ARR_FLOATS)[lane];
-        D = reinterpret_cast<const float2*>(s + 3 * ARR_FLOATS)[lane];
-        const bool rowin = k >= 0 && k < a.ny;
-        if (edge || !rowin) {
-            if (!(rowin && colA)) { E.x = U.x = V.x = 0.f; D.x = OUTSIDE_D; }
-            if (!(rowin && colB)) { E.y = U.y = V.y = 0.f; D.y = OUTSIDE_D; }
-        }
-        m = m0;
-        if (SPH && rowin) {
+    __device__ __forceinline__ XMet2 met_row(int k) const {
+        XMet2 m = m0;
+        if (SPH) {
             const float2 f = v2(__ldg(a.xrow + k));
-            m.inv_l = mul2(m.inv_l, f); m.inv_r = mul2(m.inv_r, f); m.k2 = mul2(m.k2, f);
+            m.hr = mul2(m.hr, f); m.k2 = mul2(m.k2, f);
         }
-        return rowin;
+        return m;
+    }
+    // the left intervals (the general x-sweep's walls): those of the left neighbours
+    __device__ __forceinline__ void met_left(XMet2& m) const {
+        m.hl.y = m.hr.x;
+        m.hl.x = __shfl_up_sync(FULL, m.hr.y, 1);
+        if (lane == 0) m.hl.x = m.hr.x;
     }
 
-    // the x-swept row k into the y-sweep pipeline; the finished row k - 3 goes out
+    // Whether the lane's nodes that count are wet, given their heights. EDGE: the window has
+    // columns past the domain's edge or the grid permanent walls.
+    template <bool EDGE>
+    __device__ __forceinline__ bool wet_pair(float2 H, float2 D, bool cA_, bool cB_) const {
+        float m = min_nan(H.x, H.y);
+        if (EDGE && !cB_) m = H.x;
+        bool ok = m >= K.hmin;
+        if (EDGE && a.walls) {
+            float d = min_nan(D.x, D.y);
+            if (!cB_) d = D.x;
+            ok = ok && d >= K.dwall;
+        }
+        return ok || !cA_;
+    }
+    __device__ __forceinline__ float* out_row(int r) const {
+        return O.eta_out + ((long long)b * a.plane + (long long)r * a.pitch + c0 + 2 * lane);
+    }
+
+    // Finished row r out at po, by the lanes whose nodes go out (va, vb); mw: its stored maxima
+    // in the ring (eta, then speed). EDGE: a lane's A may go out alone. MW: max-wave is due.
+    template <bool EDGE, bool MW>
+    __device__ __forceinline__ void emit(int r, float* po, bool va, bool vb, const float* mw, float2 oe, float2 ow,
+                                         float2 ot, float2 od) {
+        if (YF) {
+            // x-sweep of the y-swept row r: along-row velocity u (ot), across v (ow)
+            XMet2 m = met_row(SPH ? max(r, 0) : r);
+            const float2 H = add2(oe, od);
+            if (!S1 && __all_sync(FULL, wet_pair<EDGE>(H, od, colA, colB))) {
+                xsweep2_open<FRIC, OPEN>(oe, ot, ow, od, H, m, K, EDGE && wallx, walls, ends);
+            } else {
+                met_left(m);
+                xsweep2<FRIC, S1, OPEN>(oe, ot, ow, od, m, K, lane, ends, wallx);
+            }
+        }
+        if (vb) {
+            *reinterpret_cast<float2*>(po) = oe;
+            *reinterpret_cast<float2*>(po + a.fs_out) = ot;
+            *reinterpret_cast<float2*>(po + 2 * a.fs_out) = ow;
+            // the stored nodes only (an unstored column past the domain edge may hold anything)
+            chk_out = fma2(oe, oe, fma2(ot, ot, fma2(ow, ow, chk_out)));
+        }
+        if (EDGE) {
+            if (va && !vb) {
+                po[0] = oe.x; po[a.fs_out] = ot.x; po[2 * a.fs_out] = ow.x;
+                chk_out.x = fmaf(oe.x, oe.x, fmaf(ot.x, ot.x, fmaf(ow.x, ow.x, chk_out.x)));
+            }
+        }
+        if (MW && (MAIN || O.emax)) {
+            const float2 em = *reinterpret_cast<const float2*>(mw);
+            const float2 sm = *reinterpret_cast<const float2*>(mw + ARR_FLOATS);
+            emit_max(K, O.emax + (po - O.eta_out), a.fs_max, va, vb, oe, ot, ow, od, em, sm);
+        }
+    }
+
+    // columns past the domain's edge: at rest, dry, never wetted
+    __device__ __forceinline__ void outside(float2& E, float2& U, float2& V, float2& D) const {
+        if (!colA) { E.x = U.x = V.x = 0.f; D.x = OUTSIDE_D; }
+        if (!colB) { E.y = U.y = V.y = 0.f; D.y = OUTSIDE_D; }
+    }
+
+    // Row k in open water, at s in the ring: row k-2 in the y-sweep, row k in the x-sweep.
+    // False, with nothing done, when it is not open water.
+    template <int PH, bool EDGE, bool MW>
+    __device__ __forceinline__ bool fast_row(int k, const float* s, int kgen, float*& po) {
+        // a row before the first or after the last that counts only keeps the march going
+        const bool past = (unsigned)k > (unsigned)kpast;
+        float2 E = *reinterpret_cast<const float2*>(s + 0 * ARR_FLOATS);
+        float2 U = *reinterpret_cast<const float2*>(s + 1 * ARR_FLOATS);
+        float2 V = *reinterpret_cast<const float2*>(s + 2 * ARR_FLOATS);
+        float2 D = *reinterpret_cast<const float2*>(s + 3 * ARR_FLOATS);
+        if (YF && wallx) outside(E, U, V, D);           // its x-sweep comes later, with its votes
+        float2 H = add2(E, D);
+        bool wet = sw && (YF || past || wet_pair<EDGE>(H, D, colA, colB));
+        if (S1 || OPEN) wet = wet && k < kgen;
+        if (!__all_sync(FULL, wet)) return false;
+        const float4 q = __ldg(a.ymp + k - 2);
+        const float2 nsdt = SPH ? v2(__ldg(a.ymet + k - 2).w) : v2(0.f);
+        int edge = 0;
+        float hl = 0.f;
+        if (k == 2 || k == a.ny + 1) {
+            edge = (k == 2 ? 1 : 0) | (k == a.ny + 1 ? 2 : 0);
+            hl = __ldg(a.ymet).x;
+        }
+        float2 ne, nw, nt;
+        const float2 dP = ym.bank[PH].d;
+        ym.template fast<PH, SPH, FRIC, S1>(make_float2(q.x, q.y), make_float2(q.z, q.w), nsdt, edge, hl, K, ne, nw, nt);
+        if (!YF) {
+            XMet2 m = met_row(SPH ? min(max(k, 0), a.ny - 1) : k);
+            if (S1) {
+                met_left(m);
+                xsweep2<FRIC, S1, OPEN>(E, U, V, D, m, K, lane, ends, wallx);
+            } else {
+                xsweep2_open<FRIC, OPEN>(E, U, V, D, H, m, K, EDGE && wallx, walls, ends);
+            }
+            H = add2(E, D);
+        }
+        sw = past || wet_pair<EDGE>(H, D, YF ? colA : vA, YF ? colB : vB);
+        ym.template store_row<PH>(E, V, U, D, H);
+        const bool out = k - 2 >= r0;
+        emit<EDGE, MW>(k - 2, po, vA && out, vB && out, s + 4 * ARR_FLOATS, ne, nw, nt, dP);
+        po += a.pitch;
+        return true;
+    }
+
+    // Row k in the general case, at s in the ring when it is inside the domain (q: its row in
+    // ring slot cs). hist: rows k-2 (bit 0) and k-3 (bit 1) wet at the start of the y-sweep.
     template <int PH>
-    __device__ __forceinline__ void push_row(int k, const float* s, float2 E, float2 U, float2 V, float2 D) {
-        const float4 m2 = __ldg(a.ymet + k - 2);
-        // y-sweep input of row k: eta, w = v, t = u
-        const bool oA = wet_mark(E.x, D.x, K), oB = wet_mark(E.y, D.y, K);
+    __device__ __forceinline__ void slow_row(int k, int q, const float* s, unsigned& hist) {
+        const unsigned h1 = __all_sync(FULL, sw) ? 1u : 0u;
+        float2 E = v2(0.f), U = E, V = E, D = v2(OUTSIDE_D);
+        if (k >= 0 && k < a.ny) {
+            E = *reinterpret_cast<const float2*>(s + 0 * ARR_FLOATS);
+            U = *reinterpret_cast<const float2*>(s + 1 * ARR_FLOATS);
+            V = *reinterpret_cast<const float2*>(s + 2 * ARR_FLOATS);
+            D = *reinterpret_cast<const float2*>(s + 3 * ARR_FLOATS);
+            if (wallx) outside(E, U, V, D);
+            if (!YF) {
+                XMet2 m = met_row(k);
+                met_left(m);
+                xsweep2<FRIC, S1, OPEN>(E, U, V, D, m, K, lane, ends, wallx);
+            }
+        }
         // a non-finite x-sweep result reads as a dry node in the y-sweep and would be
-        // refilled by step (b) there: it is caught here (0 * NaN or 0 * inf is NaN)
+        // refilled by step (b) there: it is caught here (0 * NaN or 0 * inf is NaN), with that
+        // of row k-1, which the open-water x-sweep may have left (in the lanes that count)
         chk_x = fma2(E, v2(0.f), chk_x);
-        const int r = k - 3;
-        // the y-sweep results a lane must get right: its own output columns, and with YF every
-        // column of the window (the x-sweep on the way out reads three columns past the outputs)
-        ym.template push<PH, SPH, FRIC, S1, OPEN>(E, V, U, D, oA, oB, m2, K, YF ? colA : vA, YF ? colB : vB,
-            [&](float2 oe, float2 ow, float2 ot, float2 od) {
-                if (r >= r0 && r < r1) {
-                    if (YF) {
-                        // x-sweep of the y-swept row r: along-row velocity u (ot), across v (ow)
-                        XMet2 mr = m0;
-                        if (SPH) {
-                            const float2 f = v2(__ldg(a.xrow + r));
-                            mr.inv_l = mul2(mr.inv_l, f); mr.inv_r = mul2(mr.inv_r, f); mr.k2 = mul2(mr.k2, f);
-                        }
-                        xsweep2<FRIC, S1, OPEN>(oe, ot, ow, od, mr, K, lane, ends, bounded);
-                    }
-                    float2 em = make_float2(0.f, 0.f), sm = em;
-                    if (O.emax) {
-                        em = reinterpret_cast<const float2*>(s + 4 * ARR_FLOATS)[lane];
-                        sm = reinterpret_cast<const float2*>(s + 5 * ARR_FLOATS)[lane];
-                    }
-                    emit_pair<false>(a, O, orow + (size_t)(r - r0) * a.pitch, vA, vB, oe, ot, ow, od, em, sm, bad);
-                    // the stored nodes only (an unstored column past the domain edge may hold
-                    // anything after an open-water y-sweep that did not need it)
-                    const float2 q2 = fma2(oe, oe, fma2(ot, ot, mul2(ow, ow)));
-                    if (vB) chk_out = add2(chk_out, q2);
-                    else if (vA) chk_out.x += q2.x;
-                    smp.emit(a, O, b, r, c0, lane, oe, ot, ow);
-                }
-            }, OPEN ? open_end_y(a, k - 2) : 0);
+        if (vA) chk_x.x = fmaf(ym.bank[1 - PH].e.x, 0.f, chk_x.x);
+        if (vB) chk_x.y = fmaf(ym.bank[1 - PH].e.y, 0.f, chk_x.y);
+        const bool oA = wet_mark(E.x, D.x, K), oB = wet_mark(E.y, D.y, K);
+        const float4 m2 = __ldg(a.ymet + k - 2);
+        const int edge = OPEN ? open_end_y(a, k - 2) : 0;
+        ym.template slow<PH, SPH, FRIC, S1, OPEN>(E, V, U, D, oA, oB, m2, K,
+            [&](int lag, float2 oe, float2 ow, float2 ot, float2 od) {
+                const int r = k - lag;
+                if (r < r0 || r >= r1) return;
+                // the row's place among the max-wave rows, two rows ahead of the state's
+                const int qm = q + 2 - lag;
+                const float* mw = qm >= 0 ? at(cs, qm) : at(cs == 0 ? a.nslots - 1 : cs - 1, qm + SLOT_ROWS);
+                if (!MAIN || O.emax) emit<true, true>(r, out_row(r), vA, vB, mw + 4 * ARR_FLOATS, oe, ow, ot, od);
+                else emit<true, false>(r, out_row(r), vA, vB, mw, oe, ow, ot, od);
+            }, edge);
+        hist = (((ym.pend ? hist & ~1u : hist) << 1) | h1) & 3u;
+        sw = YF ? ((oA || !colA) && (oB || !colB)) : ((oA || !vA) && (oB || !vB));
     }
 
-    // row k of a ring slot: x-sweep, then into the y-sweep pipeline
-    template <int PH>
-    __device__ __forceinline__ void row(int k, const float* s) {
-        float2 E, U, V, D;
-        XMet2 m;
-        if (load_row(k, s, E, U, V, D, m) && !YF) xsweep2<FRIC, S1, OPEN>(E, U, V, D, m, K, lane, ends, bounded);
-        push_row<PH>(k, s, E, U, V, D);
-    }
-
-    // The two rows of a ring slot on Cartesian grids (x first, eq. (solver2), reflecting
-    // edges): when one vote finds every node of both rows wet, their x-sweeps run in one
-    // basic block as two independent chains (the same operations as row by row).
-    __device__ __forceinline__ void rows2(int k, const float* s) {
-        float2 E0, U0, V0, D0, E1, U1, V1, D1;
-        XMet2 m0r, m1r;
-        const bool in0 = load_row(k, s, E0, U0, V0, D0, m0r);
-        const bool in1 = load_row(k + 1, s + XWIN, E1, U1, V1, D1, m1r);
-        const bool wet = wet_mark(E0.x, D0.x, K) && wet_mark(E0.y, D0.y, K) &&
-                         wet_mark(E1.x, D1.x, K) && wet_mark(E1.y, D1.y, K);
-        if (in0 && in1 && !bounded && __all_sync(FULL, wet)) {
-            xsweep2_open<FRIC>(E0, U0, V0, D0, m0r, K);
-            xsweep2_open<FRIC>(E1, U1, V1, D1, m1r, K);
-        } else {
-            if (in0) xsweep2<FRIC, S1, OPEN>(E0, U0, V0, D0, m0r, K, lane, ends, bounded);
-            if (in1) xsweep2<FRIC, S1, OPEN>(E1, U1, V1, D1, m1r, K, lane, ends, bounded);
+    // Pairs of rows in open water from row k (row q of the slot, at s), until a row is not open
+    // water (odd: the second of its pair), the item is done (then k > r1) or a wait expires (false).
+    template <bool EDGE, bool MW>
+    __device__ __forceinline__ bool fast_rows(int& k, int& q, const float*& s, bool& odd, int kgen, int klim) {
+        float* po = out_row(k - 2);
+        while (true) {
+            if (q == SLOT_ROWS) {
+                if (!next_slot(k, __all_sync(FULL, sw))) return false;
+                q = 0;
+                s = at(cs, 0);
+            }
+            odd = false;
+            if (!fast_row<0, EDGE, MW>(k, s, kgen, po)) return true;
+            if (k > r1) { ++k; return true; }
+            if (q == 0 && k >= klim) refill(k);
+            odd = true;
+            if (!fast_row<1, EDGE, MW>(k + 1, s + XWIN, kgen, po)) return true;
+            if (q == 0 && k < klim) refill(k);
+            k += 2;
+            if (k - 1 > r1) return true;
+            q += 2;
+            s += 2 * XWIN;
         }
-        push_row<0>(k, s, E0, U0, V0, D0);
-        push_row<1>(k + 1, s + XWIN, E1, U1, V1, D1);
+    }
+
+    // General rows from row k (row q of the slot, at s; odd: from the second of its pair) up to
+    // the next pair after three rows of open water, the end of the item (k - 1 > r1) or an
+    // expired wait (false).
+    __device__ __forceinline__ bool slow_rows(int& k, int& q, const float*& s, bool odd, unsigned hist, int kgen) {
+        while (true) {
+            if (!odd) {
+                if (q == SLOT_ROWS) {
+                    if (!next_slot(k, false)) return false;
+                    q = 0;
+                    s = at(cs, 0);
+                }
+                slow_row<0>(k, q, s, hist);
+                if (k > r1 && (!ym.pend || k == r1 + 2)) { ++k; return true; }
+                if (q == 0 && k != k0) refill(k);
+            }
+            odd = false;
+            slow_row<1>(k + 1, q + 1, s + XWIN, hist);
+            const bool done = k >= r1 && (!ym.pend || k + 1 == r1 + 2);
+            if (!done && q == 0 && k != k0) refill(k);
+            k += 2;
+            q += 2;
+            s += 2 * XWIN;
+            if (done || (hist == 3u && k < kgen && __all_sync(FULL, sw))) return true;
+        }
     }
 
     // Process work item `idx` (strip, rows) of scenario b_ for the step described by O_.
     // Returns false when a wait expired (the warp's copies have landed when it returns).
     __device__ __forceinline__ bool run_item(int idx, int b_, const StepOut& O_) {
         O = O_;
-        b = b_;
+        b = uniform(b_);
         const int4 item = __ldg(a.items + idx);          // (strip, first row, end row)
-        c0 = item.x * XOUT;                          // window columns c0 .. c0 + 63 (fused_strips)
-        cA = c0 + 2 * lane;
-        r0 = item.y;
-        r1 = item.z;
+        c0 = uniform(item.x) * XOUT;                          // window columns c0 .. c0 + 63 (fused_strips)
+        const int cA = c0 + 2 * lane;
+        r0 = uniform(item.y);
+        r1 = uniform(item.z);
         k0 = r0 - 3;
-        npairs = (r1 + 3 - k0 + 1) / 2;
-        orow = (size_t)b * a.plane + (size_t)r0 * a.pitch + cA;
-        nbox = O.emax ? 6u : 4u;
-        tx = nbox * ARR_FLOATS * 4u + a.tx_pad;
-        colA = cA >= 0 && cA < a.nx;
-        ends = OPEN ? open_ends_x(a, cA) : 0u;
-        colB = cA + 1 >= 0 && cA + 1 < a.nx;
+        kpast = min(r1, a.ny - 1);
+        tx = (O.emax ? 6u : 4u) * ARR_FLOATS * 4u + a.tx_pad;
+        colA = cA < a.nx;
+        colB = cA + 1 < a.nx;
         // the output columns: c0 + 4 .. c0 + 59, and from the domain's first column in the
         // first window, to its last column in the window that reaches it (past it the
         // window holds dry ghost columns, or its edge is the domain's)
         const bool own = (lane >= 2 || c0 == 0) && (lane < 30 || c0 + XWIN >= a.nx);
         vA = own && colA;
         vB = own && colB;
-        edge = c0 + XWIN > a.nx;
-        bounded = c0 == 0 || c0 + XWIN == a.nx;
-        for (int j = 0; j < min(RING, npairs); ++j) issue(j);
-        float2 il = v2(0.f), ir = v2(0.f), k2 = v2(0.f);
-        if (colA) { il.x = __ldg(a.xa + cA); ir.x = __ldg(a.xb + cA); k2.x = __ldg(a.xk + cA); }
-        if (colB) { il.y = __ldg(a.xa + cA + 1); ir.y = __ldg(a.xb + cA + 1); k2.y = __ldg(a.xk + cA + 1); }
-        m0 = XMet2{il, ir, k2};
-        smp.init(a, O, idx, lane);
+        wallx = c0 == 0 || c0 + XWIN >= a.nx;
+        walls = wall_ends_x(cA, a.nx);
+        ends = OPEN ? open_ends_x(a, cA) : 0u;
+        // the slots the open-water march reads (with max-wave due its rows count too)
+        ntot = ((O.emax ? r1 + 1 : kpast) - k0) / SLOT_ROWS + 1;
+        nfill = nread = 0;
+        cs = head;
+        const int first = head;
+        while (nfill < min(a.nslots, ntot)) fill();
+        float2 hr = v2(0.f), k2 = v2(0.f);
+        if (colA) { hr.x = __ldg(a.xb + cA); k2.x = __ldg(a.xk + cA); }
+        if (colB) { hr.y = __ldg(a.xb + cA + 1); k2.y = __ldg(a.xk + cA + 1); }
+        m0 = XMet2{v2(0.f), hr, k2};
         ym.init();
-        int j = 0;
-        for (; j < npairs; ++j) {
-            const int slot = (int)((used + (unsigned)j) % RING);
-            const bool ok = mbar_wait(&bar[slot], ((used + (unsigned)j) / RING) & 1u, a.wait_cycles);
-            if (!__all_sync(FULL, ok)) break;
-            const float* s = ring + slot * SLOT_FLOATS;
-            const int k = k0 + SLOT_ROWS * j;
-            if (!SPH && !YF && !S1 && !OPEN) {
-                rows2(k, s);
-            } else {
-                row<0>(k, s);
-                row<1>(k + 1, s + XWIN);
+        // An open first or last row and eq. (solver1)'s flux around one take the general path: no
+        // open water from row kgen on, and no start in open water above row 0.
+        const int kgen = ((OPEN && (a.open_edges & 8) != 0) || S1) ? a.ny - 1 : 0x7fffffff;
+        bool opt = !(((OPEN && (a.open_edges & 4) != 0) || S1) && r0 == 0);
+        // the last row whose vote may still send the march back to row r0-3: a general row k
+        // needs the flux (k-3 | k-2), or the wall above row 0, from the rows before it
+        const int klim = r0 == 0 ? 2 : r0 + 1;
+        int k = opt ? r0 - 1 : k0, q = k - k0;
+        unsigned hist = 0u;
+        sw = opt;
+        bool ok = acquire(), odd = false;
+        const float* s = at(cs, q);
+        bool fast = opt;
+        while (ok) {
+            if (fast) {
+                if (!MAIN)
+                    ok = fast_rows<true, true>(k, q, s, odd, kgen, klim);
+                else if (wallx || a.walls)
+                    ok = O.emax ? fast_rows<true, true>(k, q, s, odd, kgen, klim) : fast_rows<true, false>(k, q, s, odd, kgen, klim);
+                else
+                    ok = O.emax ? fast_rows<false, true>(k, q, s, odd, kgen, klim) : fast_rows<false, false>(k, q, s, odd, kgen, klim);
+                if (!ok || k - 1 > r1) break;
+                ym.after_fast();
+                hist = 3u;
+                if (opt && k + (odd ? 1 : 0) <= klim) {     // start over from row r0-3
+                    k = k0;
+                    q = 0;
+                    cs = first;
+                    s = at(cs, 0);
+                    odd = false;
+                    hist = 0u;
+                    sw = false;
+                    ym.init();
+                }
+                opt = false;
             }
-            __syncwarp();
-            if (j + RING < npairs) issue(j + RING);
+            ok = slow_rows(k, q, s, odd, hist, kgen);
+            if (!ok || k - 1 > r1) break;
+            odd = false;
+            fast = true;
         }
-        if (j < npairs) {
-            // a wait expired at pair j: pairs j .. j+RING-1 may still be in flight; let
-            // each land (bounded) before going on
-            for (int i = j; i < min(j + RING, npairs); ++i)
-                mbar_wait(&bar[(used + (unsigned)i) % RING], ((used + (unsigned)i) / RING) & 1u, a.wait_cycles);
+        if (!ok) {
+            // a wait expired: the slots filled may still be in flight; let each land (bounded)
+            // before going on
+            for (; nread < nfill; ++nread) {
+                mbar_wait(&bar[cs], (phase >> cs) & 1u, a.wait_cycles);
+                cs = next_of(cs);
+            }
             bad |= 2;
             return false;
         }
-        used += (unsigned)npairs;
+        write_samples(a, O, idx, b, lane);
         return true;
     }
 
@@ -441,15 +596,15 @@ struct FusedWarp {
 
 template <bool SPH, bool FRIC, bool YF, bool S1, bool OPEN>
 __global__ void __launch_bounds__(FUSED_WARPS * 32, 4)
-k_step_fused(const __grid_constant__ StepMaps M, const StepArgs a) {
+k_step_fused(const __grid_constant__ StepMaps M, const __grid_constant__ StepArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int wib = threadIdx.x >> 5;
-    const int gw = blockIdx.x * FUSED_WARPS + wib;
+    const int gw = uniform(blockIdx.x * FUSED_WARPS + wib);
     const int b = blockIdx.y;
     if (gw >= a.nitems) return;
-    if (a.limit && a.step > a.limit[b]) return;
+    if (a.limit && __all_sync(FULL, a.step > a.limit[b])) return;
     // a wait of an earlier launch expired: do not start new copies
-    if (*reinterpret_cast<volatile int*>(a.err) & ERRF_TIMEOUT) return;
+    if (__any_sync(FULL, *reinterpret_cast<volatile int*>(a.err) & ERRF_TIMEOUT)) return;
     FusedWarp<SPH, FRIC, YF, S1, OPEN> W(a);
     W.setup(smem_raw, wib);
     W.run_item(gw, b, step_out(&M, a));
@@ -499,10 +654,10 @@ __device__ __forceinline__ bool grid_sync(unsigned long long* bar, unsigned nblo
 // uses while the other is in use. A scenario that has stopped keeps its last state in the
 // buffer of its last step's parity.
 // With ALT (the alternating order) the odd-indexed steps (st - 1 odd) sweep y first: a second
-// per-warp worker of the y-first kind shares the warp's ring, barriers and ring count.
+// per-warp worker of the y-first kind shares the warp's ring, barriers and ring position.
 template <bool SPH, bool FRIC, bool S1, bool OPEN, bool ALT>
 __global__ void __launch_bounds__(FUSED_WARPS * 32, 4)
-k_batch(const __grid_constant__ StepMaps2 MM, const StepArgs a, const BatchArgs B) {
+k_batch(const __grid_constant__ StepMaps2 MM, const __grid_constant__ StepArgs a, const __grid_constant__ BatchArgs B) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int wib = threadIdx.x >> 5;
     const long long step0 = B.ctl[0], step_end = B.ctl[1];
@@ -512,19 +667,19 @@ k_batch(const __grid_constant__ StepMaps2 MM, const StepArgs a, const BatchArgs 
     W.setup(smem_raw, wib);
     FusedWarp<SPH, FRIC, true, S1, OPEN> WY(a);
     if (ALT) {
-        WY.lane = W.lane; WY.K = W.K; WY.ring = W.ring; WY.bar = W.bar; WY.used = W.used; WY.bad = 0;
+        WY.lane = W.lane; WY.ring = W.ring; WY.bar = W.bar; WY.bad = 0;
         WY.chk_x = WY.chk_out = v2(0.f);
     }
     for (long long st = step0 + 1; st <= step_end; ++st) {
         const bool yf = ALT && (((st - 1) & 1) != 0);
-        if (yf) WY.used = W.used;
+        if (yf) { WY.head = W.head; WY.phase = W.phase; }
         if (B.bnd) {
             // boundary input: the edge nodes of this step's input take the input at its model
             // time, then every block waits so that no TMA load reads an edge before it is set
             const BndRow& R = B.bnd_rows[st - step0 - 1];
             float* ei = (st & 1) ? B.eta[0] : B.eta[1];
-            float* ui = (st & 1) ? B.u[0] : B.u[1];
-            float* vi = (st & 1) ? B.v[0] : B.v[1];
+            float* ui = ei + a.fs_out;
+            float* vi = ei + 2 * a.fs_out;
             const int per = 2 * a.ny + 2 * a.nx;
             for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < per; idx += gridDim.x * blockDim.x) {
                 const int e = idx < a.ny ? 0 : idx < 2 * a.ny ? 1 : idx < 2 * a.ny + a.nx ? 2 : 3;
@@ -535,8 +690,7 @@ k_batch(const __grid_constant__ StepMaps2 MM, const StepArgs a, const BatchArgs 
         }
         const bool odd = (st & 1) != 0;          // odd steps read buffer 0 and write buffer 1
         const bool mx = st % B.maxout == 0;
-        StepOut O{odd ? &MM.m[0] : &MM.m[1], odd ? B.eta[1] : B.eta[0], odd ? B.u[1] : B.u[0],
-                  odd ? B.v[1] : B.v[0], mx ? B.emax : nullptr, mx ? B.smax : nullptr,
+        StepOut O{odd ? &MM.m[0] : &MM.m[1], odd ? B.eta[1] : B.eta[0], mx ? B.emax : nullptr,
                   (B.grec && st % B.gout == 0) ? B.grec + (st / B.gout) * B.grec_row : nullptr,
                   (B.nrec && st % B.bndout == 0) ? B.nrec + (st / B.bndout) * B.nrec_row : nullptr};
         const int na = B.nact ? (st < B.nact_len ? __ldg(B.nact + st) : 0) : B.nall;
@@ -546,12 +700,12 @@ k_batch(const __grid_constant__ StepMaps2 MM, const StepArgs a, const BatchArgs 
         while (ok) {
             unsigned t = 0;
             if (W.lane == 0) t = atomicAdd(tickets + (odd ? 1 : 0), 1u);
-            t = __shfl_sync(FULL, t, 0);
+            t = (unsigned)uniform((int)__shfl_sync(FULL, t, 0));
             if (t >= total) break;
-            const int item = (int)(t % (unsigned)a.nitems), scen = __ldg(B.order + t / (unsigned)a.nitems);
+            const int item = (int)(t % (unsigned)a.nitems), scen = uniform(__ldg(B.order + t / (unsigned)a.nitems));
             ok = yf ? WY.run_item(item, scen, O) : W.run_item(item, scen, O);
         }
-        if (yf) W.used = WY.used;
+        if (yf) { W.head = WY.head; W.phase = WY.phase; }
         if (!ok && W.lane == 0) atomicOr(a.err, ERRF_TIMEOUT);
         if (!grid_sync(reinterpret_cast<unsigned long long*>(B.ctl + 2), gridDim.x, a.wait_cycles, a.err)) break;
     }
@@ -571,32 +725,30 @@ __global__ void __launch_bounds__(128) k_xsweep(const StepArgs a) {
     const int c0 = strip * XOUT - 4;
     const int cA = c0 + 2 * lane;
     const size_t boff = (size_t)b * a.plane;
-    const SweepConst K{a.hmin, a.dwall, a.half_dt, a.dt_gn2, a.transverse, a.inv_dt2_s1};
+    const SweepConst& K = a.K;
     float2 il = v2(0.f), ir = v2(0.f), k2 = v2(0.f);
     if (cA >= 0 && cA < a.nx) { il.x = a.xa[cA]; ir.x = a.xb[cA]; k2.x = a.xk[cA]; }
     if (cA + 1 >= 0 && cA + 1 < a.nx) { il.y = a.xa[cA + 1]; ir.y = a.xb[cA + 1]; k2.y = a.xk[cA + 1]; }
     XMet2 m{il, ir, k2};
     if (SPH) {
         const float2 f = v2(a.xrow[r]);
-        m.inv_l = mul2(m.inv_l, f); m.inv_r = mul2(m.inv_r, f); m.k2 = mul2(m.k2, f);
+        m.hl = mul2(m.hl, f); m.hr = mul2(m.hr, f); m.k2 = mul2(m.k2, f);
     }
     float2 E, U, V, D;
     load_pair(a, boff, r, cA, E, U, V, D);
     xsweep2<FRIC, S1, OPEN>(E, U, V, D, m, K, lane, OPEN ? open_ends_x(a, cA) : 0u);
     const bool own = lane >= 2 && lane < 30;
     const bool va = own && cA < a.nx, vb = own && cA + 1 < a.nx;
-    int bad = 0;
     const size_t o = boff + (size_t)r * a.pitch + cA;
-    float2 em = make_float2(0.f, 0.f), sm = em;
     const StepOut O = step_out(nullptr, a);
+    emit_pair(a.eta_out + o, a.fs_out, va, vb, E, U, V);
+    int bad = (va && runaway(E.x, U.x, V.x)) | (vb && runaway(E.y, U.y, V.y));
     if (O.emax && va) {
-        em.x = a.emax[o]; sm.x = a.smax[o];
-        if (vb) { em.y = a.emax[o + 1]; sm.y = a.smax[o + 1]; }
+        float2 em = make_float2(a.emax[o], 0.f), sm = make_float2(a.emax[o + a.fs_max], 0.f);
+        if (vb) { em.y = a.emax[o + 1]; sm.y = a.emax[o + 1 + a.fs_max]; }
+        emit_max(a.K, a.emax + o, a.fs_max, va, vb, E, U, V, D, em, sm);
     }
-    emit_pair(a, O, o, va, vb, E, U, V, D, em, sm, bad);
-    Samples smp;
-    smp.init(a, O, gw, lane);
-    smp.emit(a, O, b, r, c0, lane, E, U, V);
+    write_samples(a, O, gw, b, lane);
     if (bad) atomicOr(a.err, ERRF_NONFINITE);
 }
 
@@ -604,35 +756,46 @@ __global__ void __launch_bounds__(128) k_xsweep(const StepArgs a) {
 template <bool SPH, bool FRIC, bool S1, bool OPEN>
 struct YOnly {
     const StepArgs& a;
-    SweepConst K;
+    const SweepConst& K;
     int lane, b, c0, cA, r0, r1;
     size_t boff;
-    bool vA, vB, withmax;
+    bool vA, vB;
+    unsigned hist;             // rows k-1, k-2, k-3 (bits 0-2) wet at the start of the sweep
     YMarch2 ym;
-    Samples smp;
     StepOut O;
     int bad;
-    __device__ __forceinline__ YOnly(const StepArgs& a_) : a(a_) {}
+    __device__ __forceinline__ YOnly(const StepArgs& a_) : a(a_), K(a_.K) {}
+    __device__ __forceinline__ void emit(int r, float2 oe, float2 ow, float2 ot, float2 od) {
+        if (r < r0 || r >= r1) return;
+        const size_t o = boff + (size_t)r * a.pitch + cA;
+        emit_pair(a.eta_out + o, a.fs_out, vA, vB, oe, ot, ow);
+        bad |= (vA && runaway(oe.x, ot.x, ow.x)) | (vB && runaway(oe.y, ot.y, ow.y));
+        if (O.emax && vA) {
+            float2 em = make_float2(a.emax[o], 0.f), sm = make_float2(a.emax[o + a.fs_max], 0.f);
+            if (vB) { em.y = a.emax[o + 1]; sm.y = a.emax[o + 1 + a.fs_max]; }
+            emit_max(K, a.emax + o, a.fs_max, vA, vB, oe, ot, ow, od, em, sm);
+        }
+    }
     template <int PH>
     __device__ __forceinline__ void row(int k) {
         float2 E, U, V, D;
         load_pair(a, boff, k, cA, E, U, V, D);
         const float4 m2 = __ldg(a.ymet + k - 2);
         const bool oA = wet_mark(E.x, D.x, K), oB = wet_mark(E.y, D.y, K);
-        const int r = k - 3;
-        ym.template push<PH, SPH, FRIC, S1, OPEN>(E, V, U, D, oA, oB, m2, K, vA, vB,
-            [&](float2 oe, float2 ow, float2 ot, float2 od) {
-                if (r >= r0 && r < r1) {
-                    const size_t o = boff + (size_t)r * a.pitch + cA;
-                    float2 em = make_float2(0.f, 0.f), sm = em;
-                    if (O.emax && vA) {
-                        em.x = a.emax[o]; sm.x = a.smax[o];
-                        if (vB) { em.y = a.emax[o + 1]; sm.y = a.smax[o + 1]; }
-                    }
-                    emit_pair(a, O, o, vA, vB, oe, ot, ow, od, em, sm, bad);
-                    smp.emit(a, O, b, r, c0, lane, oe, ot, ow);
-                }
-            }, OPEN ? open_end_y(a, k - 2) : 0);
+        if (hist == 7u) {
+            float2 ne, nw, nt;
+            const float2 dP = ym.bank[PH].d;
+            ym.template fast<PH, SPH, FRIC, S1>(v2(m2.y), v2(m2.z), v2(m2.w), 0, 0.f, K, ne, nw, nt);
+            ym.template store_row<PH>(E, V, U, D, add2(E, D));
+            ym.after_fast();
+            emit(k - 2, ne, nw, nt, dP);
+        } else {
+            ym.template slow<PH, SPH, FRIC, S1, OPEN>(E, V, U, D, oA, oB, m2, K,
+                [&](int lag, float2 oe, float2 ow, float2 ot, float2 od) { emit(k - lag, oe, ow, ot, od); },
+                OPEN ? open_end_y(a, k - 2) : 0);
+            if (ym.pend) hist &= ~2u;                  // row k-2 waits for its (e)
+        }
+        hist = ((hist << 1) | (__all_sync(FULL, (oA || !vA) && (oB || !vB)) ? 1u : 0u)) & 7u;
     }
 };
 
@@ -644,7 +807,6 @@ __global__ void __launch_bounds__(128) k_ysweep(const StepArgs a) {
     if (gw >= a.nstrips * a.nseg) return;
     if (a.limit && a.step > a.limit[b]) return;
     YOnly<SPH, FRIC, S1, OPEN> Y(a);
-    Y.K = SweepConst{a.hmin, a.dwall, a.half_dt, a.dt_gn2, a.transverse, a.inv_dt2_s1};
     const int strip = gw % a.nstrips, seg = gw / a.nstrips;
     Y.lane = lane;
     Y.b = b;
@@ -655,10 +817,9 @@ __global__ void __launch_bounds__(128) k_ysweep(const StepArgs a) {
     Y.boff = (size_t)b * a.plane;
     Y.vA = Y.cA < a.nx;
     Y.vB = Y.cA + 1 < a.nx;
-    Y.withmax = a.emax != nullptr;
+    Y.hist = 0u;
     Y.bad = 0;
     Y.O = step_out(nullptr, a);
-    Y.smp.init(a, Y.O, gw, lane);
     Y.ym.init();
     int k = Y.r0 - 3;
     for (; k + 1 < Y.r1 + 3; k += 2) {
@@ -666,6 +827,7 @@ __global__ void __launch_bounds__(128) k_ysweep(const StepArgs a) {
         Y.template row<1>(k + 1);
     }
     if (k < Y.r1 + 3) Y.template row<0>(k);
+    write_samples(a, Y.O, gw, b, lane);
     if (Y.bad) atomicOr(a.err, ERRF_NONFINITE);
 }
 

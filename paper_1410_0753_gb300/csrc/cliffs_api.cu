@@ -292,6 +292,15 @@ void cliffs::set_last_error(const char* msg) {
 
 // ----------------------------------------------------------------------------- grid
 
+// Work items of one kernel: (strip, first row, end row, 0), and per item the gauge / enclosed-
+// grid samples in it (CSR).
+struct ItemSet {
+    std::vector<int4> items;
+    int4* dev = nullptr;
+    int* samp_ptr = nullptr;
+    int4* samp = nullptr;
+};
+
 struct cliffs_grid {
     cliffs_config cfg{};
     std::vector<int32_t> gauges;
@@ -322,8 +331,6 @@ struct cliffs_grid {
     std::vector<int4> samples;
     int G = 0, NN = 0;
     int4* items_d = nullptr;
-    int* samp_ptr = nullptr;
-    int4* samp = nullptr;
     // records
     float* grec = nullptr;
     long long grec_cap = 0;
@@ -340,8 +347,9 @@ struct cliffs_grid {
     int S = 32, nstrips = 0, nseg = 0;
     std::vector<unsigned char> hard;         // [nstrips][ny]: dry nodes in the strip's window within 3 rows
     std::vector<double> strip_cost;          // per strip: the cost of its rows (item_cost)
-    std::vector<int4> items;                 // fused kernel work items (strip, r0, r1, 0)
-    int4* items_dev = nullptr;
+    ItemSet march, tile;                     // work items of the fused kernel (1D: samples only) and of the tiles
+    int tile_R = 0, tile_rows = 0;           // rows per tile in open water; the largest tile with its halo
+    bool S_set = false;                      // S was set or tuned by the caller: steps march
     // timing
     bool timing = false;
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev;
@@ -362,7 +370,7 @@ struct cliffs_grid {
     cudaStream_t cap = nullptr;
     cudaGraphExec_t gexec = nullptr;
     std::vector<unsigned char> gkey;
-    int pblocks = 0;
+    int pblocks = 0, pblocks_tile = 0;
     // adjoint work space: K recomputed states of up to adj_G segments ([3][adj_G][plane]
     // per state) and the checkpoints (row-major, 3 planes each), the transposed x-swept
     // state, adjoint and depth (7 planes of [nx][tpitch]), the row-major intermediate
@@ -439,27 +447,29 @@ long long steps_of(const cliffs_grid* g, int b) {
 int fused_strips(int nx) { return nx <= XWIN ? 1 : (nx - XWIN + XOUT - 1) / XOUT + 1; }
 int fused_strip_of(int c, int nstrips) { return c < XOUT + 4 ? 0 : std::min((c - 4) / XOUT, nstrips - 1); }
 
-// per-warp sample lists for the current launch geometry
-int build_samples(cliffs_grid* g) {
+// sample lists of an item set for the current launch geometry
+int build_samples(cliffs_grid* g, ItemSet& set) {
     // a warp owns output columns [W * strip, W * strip + W): 56 for the x-sweep alone, 64 for
     // the y-sweep alone; the fused kernels' strips are those of fused_strips
     const int W = (g->kind == 2) ? XWIN : XOUT;
     const int S = g->kind == 1 ? 1 : g->S;
     const int nseg = g->kind == 1 ? g->ny : g->nseg;
     long long nw = (long long)g->nstrips * nseg;
-    // kind 0: warp index of (row, strip) from the item table
+    // kind 0: item of (row, strip) from the item table
     std::vector<std::vector<int>> seg_start;
     std::vector<std::vector<int>> seg_item;
     if (g->kind == 0) {
-        nw = (long long)g->items.size();
-        seg_start.assign(g->nstrips, {});
-        seg_item.assign(g->nstrips, {});
-        for (size_t i = 0; i < g->items.size(); ++i) {
-            seg_start[g->items[i].x].push_back(g->items[i].y);
-            seg_item[g->items[i].x].push_back((int)i);
+        nw = (long long)set.items.size();
+        if (!g->samples.empty()) {
+            seg_start.assign(g->nstrips, {});
+            seg_item.assign(g->nstrips, {});
+            for (size_t i = 0; i < set.items.size(); ++i) {
+                seg_start[set.items[i].x].push_back(set.items[i].y);
+                seg_item[set.items[i].x].push_back((int)i);
+            }
         }
     }
-    std::vector<std::vector<int4>> per(nw);
+    std::vector<std::vector<int4>> per(g->samples.empty() ? 0 : nw);
     for (const int4& it : g->samples) {
         long long w;
         if (g->kind == 0) {
@@ -472,25 +482,22 @@ int build_samples(cliffs_grid* g) {
         }
         per[w].push_back(it);
     }
+    cudaFree(set.samp_ptr);
+    cudaFree(set.samp);
+    set.samp_ptr = nullptr;
+    set.samp = nullptr;
+    if (per.empty()) return CLIFFS_OK;
     std::vector<int> ptr(nw + 1, 0);
     std::vector<int4> flat;
     for (long long w = 0; w < nw; ++w) {
-        std::stable_sort(per[w].begin(), per[w].end(),
-                         [](const int4& a, const int4& b) { return a.x < b.x; });
         ptr[w] = (int)flat.size();
         flat.insert(flat.end(), per[w].begin(), per[w].end());
     }
     ptr[nw] = (int)flat.size();
-    if (g->samp_ptr) CK(cudaFree(g->samp_ptr));
-    if (g->samp) CK(cudaFree(g->samp));
-    g->samp_ptr = nullptr;
-    g->samp = nullptr;
-    CK(cudaMalloc(&g->samp_ptr, sizeof(int) * (nw + 1)));
-    CK(cudaMemcpy(g->samp_ptr, ptr.data(), sizeof(int) * (nw + 1), cudaMemcpyHostToDevice));
-    if (!flat.empty()) {
-        CK(cudaMalloc(&g->samp, sizeof(int4) * flat.size()));
-        CK(cudaMemcpy(g->samp, flat.data(), sizeof(int4) * flat.size(), cudaMemcpyHostToDevice));
-    }
+    CK(cudaMalloc(&set.samp_ptr, sizeof(int) * (nw + 1)));
+    CK(cudaMemcpy(set.samp_ptr, ptr.data(), sizeof(int) * (nw + 1), cudaMemcpyHostToDevice));
+    CK(cudaMalloc(&set.samp, sizeof(int4) * flat.size()));
+    CK(cudaMemcpy(set.samp, flat.data(), sizeof(int4) * flat.size(), cudaMemcpyHostToDevice));
     return CLIFFS_OK;
 }
 
@@ -524,17 +531,28 @@ void cut_items(const cliffs_grid* g, int S, std::vector<int4>& items) {
     }
 }
 
+int upload_items(cliffs_grid* g, ItemSet& set) {
+    cudaFree(set.dev);
+    set.dev = nullptr;
+    CK(cudaMalloc(&set.dev, sizeof(int4) * set.items.size()));
+    CK(cudaMemcpy(set.dev, set.items.data(), sizeof(int4) * set.items.size(), cudaMemcpyHostToDevice));
+    return build_samples(g, set);
+}
+
 int set_rows_per_warp(cliffs_grid* g, int S) {
     g->S = S;
     g->nseg = (g->ny + S - 1) / S;
-    if (g->kind == 0) {
-        cut_items(g, S, g->items);
-        cudaFree(g->items_dev);
-        g->items_dev = nullptr;
-        CK(cudaMalloc(&g->items_dev, sizeof(int4) * g->items.size()));
-        CK(cudaMemcpy(g->items_dev, g->items.data(), sizeof(int4) * g->items.size(), cudaMemcpyHostToDevice));
-    }
-    return build_samples(g);
+    if (g->kind != 0) return build_samples(g, g->march);
+    cut_items(g, S, g->march.items);
+    return upload_items(g, g->march);
+}
+
+int set_tile_rows(cliffs_grid* g, int R) {
+    cut_items(g, R, g->tile.items);
+    g->tile_R = R;
+    g->tile_rows = 0;
+    for (const int4& it : g->tile.items) g->tile_rows = std::max(g->tile_rows, it.z - it.y + 6);
+    return upload_items(g, g->tile);
 }
 
 // warps of one fused launch with S rows per warp, and the warps resident at once
@@ -545,12 +563,14 @@ long long fused_warps(const cliffs_grid* g, int S) {
     return n * g->B;
 }
 
-long long resident_warps(const cliffs_grid* g) {
+int num_sms() {
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    return (long long)std::max(1, nsm) * std::max(1, fused_blocks_per_sm(g->cfg.coords != 1)) *
-           fused_warps_per_block();
+    return std::max(1, nsm);
+}
+long long resident_warps(const cliffs_grid* g) {
+    return (long long)num_sms() * std::max(1, fused_blocks_per_sm(g->cfg.coords != 1)) * fused_warps_per_block();
 }
 
 // the smallest even S whose launch fits in `waves` waves of resident warps (0 if none does)
@@ -577,6 +597,33 @@ double launch_cost(int S, long long n, long long resident, long long nsched) {
     return (S + 3.7) * (full + last[q]);
 }
 
+// Rows per tile: the smallest modelled time of a launch of the tile kernel. A block's time is
+// its warps' share of the tile's x-sweeps and y-sweeps (rounded up to whole rows per warp) and a
+// constant; blocks come in rounds of the resident ones, two to an SM.
+int choose_tile(cliffs_grid* g) {
+    const long long resident = (long long)num_sms() * 2;
+    const int W = tile_warps_per_block(), rmax = std::min(tile_max_rows() - 6, std::max(1, g->ny));
+    double best = 1e300;
+    int bestR = rmax;
+    for (int R = 1; R <= rmax; ++R) {
+        const long long n = fused_warps(g, R);
+        const long long rounds = (n + resident - 1) / resident;
+        // one block alone on an SM runs faster than two
+        const double share = rounds == 1 && 2 * n <= resident ? 0.6 : 1.0;
+        const double cost = rounds * (share * ((R + 6 + W - 1) / W + (R + W - 1) / W) + 3.0);
+        if (cost < best) { best = cost; bestR = R; }
+    }
+    return set_tile_rows(g, bestR);
+}
+
+// Whether steps go by tiles: when every tile of a step is resident at once (up to about 1.4 M
+// nodes). Measured per step, tiles against marching warps: 200^2 beach 8.5 and 12.6 us, 512^2 10.5 and
+// 16.7, 1024^2 19.3 and 23.0, 1201 x 901 25.7 and 29.8; beyond one round the tiles' loads and
+// shared-memory traffic cost more (2048^2 geographic 91 and 60 us).
+bool by_tiles(const cliffs_grid* g) {
+    return g->kind == 0 && !g->S_set && (long long)g->tile.items.size() * g->B <= 2ll * num_sms();
+}
+
 int choose_geometry(cliffs_grid* g) {
     if (g->ny == 1) {
         g->kind = 1;
@@ -601,9 +648,12 @@ int choose_geometry(cliffs_grid* g) {
             const double cost = launch_cost(S, fused_warps(g, S), resident, nsched);
             if (cost <= best) { best = cost; bestS = S; }
         }
-        return set_rows_per_warp(g, bestS);
+        const int rc = set_rows_per_warp(g, bestS);
+        if (rc) return rc;
+        g->S_set = false;
+        return choose_tile(g);
     }
-    return build_samples(g);
+    return build_samples(g, g->march);
 }
 
 int grow_records(cliffs_grid* g, long long need_g, long long need_n) {
@@ -688,20 +738,30 @@ int make_maps(cliffs_grid* g) {
     return CLIFFS_OK;
 }
 
+// the step by tiles in place of marching warps
+void use_tiles(const cliffs_grid* g, StepArgs& a) {
+    a.items = g->tile.dev;
+    a.nitems = (int)g->tile.items.size();
+    a.samp_ptr = g->tile.samp_ptr;
+    a.samp = g->tile.samp;
+}
+
 void fill_step_args(cliffs_grid* g, StepArgs& a, int in, int out) {
     a.eta_in = g->eta[in]; a.u_in = g->u[in]; a.v_in = g->v[in];
+    a.fs_in = (long long)g->B * g->plane;
     a.eta_out = g->eta[out];
     a.fs_out = a.fs_max = (long long)g->B * g->plane;
     a.d = g->d32;
     a.xa = g->xa; a.xb = g->xb; a.xk = g->xk; a.xrow = g->xrow + MET_PAD; a.ymet = g->ymet + MET_PAD; a.ymp = g->ymp + MET_PAD;
     a.emax = nullptr; a.rec_g = nullptr; a.rec_n = nullptr;
     a.rec_g_bstride = g->grec_cap * g->G * 3;
-    a.samp_ptr = g->samp_ptr; a.samp = g->samp;
+    a.samp_ptr = g->march.samp_ptr; a.samp = g->march.samp;
     a.limit = g->limit;
     a.err = g->err;
     a.nx = g->nx; a.ny = g->ny; a.pitch = g->pitch; a.plane = g->plane;
     a.S = g->S; a.nstrips = g->nstrips; a.nseg = g->nseg;
-    a.items = g->items_dev; a.nitems = (int)g->items.size();
+    a.items = g->march.dev; a.nitems = (int)g->march.items.size();
+    a.tile_rows = g->tile_rows;
     const double gn2 = g->cfg.dt * 9.81 * g->cfg.manning_n2;
     a.K.hmin = (float)g->cfg.h_min;
     a.K.dwall = g->cfg.itopo ? -3.402823466e38f : (float)g->cfg.dwall;
@@ -822,8 +882,9 @@ void free_grid(cliffs_grid* g) {
     cudaFree(g->d32); cudaFree(g->d64); cudaFree(g->d64b);
     cudaFree(g->emax);
     cudaFree(g->xa); cudaFree(g->xb); cudaFree(g->xk); cudaFree(g->xrow); cudaFree(g->ymet); cudaFree(g->ymp);
-    cudaFree(g->err); cudaFree(g->limit); cudaFree(g->items_d); cudaFree(g->items_dev);
-    cudaFree(g->samp_ptr); cudaFree(g->samp); cudaFree(g->grec); cudaFree(g->nrec);
+    cudaFree(g->err); cudaFree(g->limit); cudaFree(g->items_d);
+    for (ItemSet* t : {&g->march, &g->tile}) { cudaFree(t->dev); cudaFree(t->samp_ptr); cudaFree(t->samp); }
+    cudaFree(g->grec); cudaFree(g->nrec);
     cudaFree(g->pt_slot); cudaFree(g->pt_w); cudaFree(g->tmp); cudaFree(g->ured);
     cudaFree(g->order_d); cudaFree(g->nact_d); cudaFree(g->ctl_d);
     if (g->ctl_h) cudaFreeHost(g->ctl_h);
@@ -1359,6 +1420,7 @@ int cliffs_step_n(cliffs_grid* g, int64_t n) {
     if (rc) return rc;
     cudaStream_t s = g->stream;
     StepArgs a;
+    const bool tiles = by_tiles(g) && g->inject_cycles <= 0;
     const double t_end = g->bnd_any ? bnd_end(g) : 1e300;
     for (long long k = 0; k < n; ++k) {
         const long long st = g->step + 1;
@@ -1389,7 +1451,10 @@ int cliffs_step_n(cliffs_grid* g, int64_t n) {
             CK(cudaEventRecord(e0, s));
         }
         cudaError_t le;
-        if (g->kind == 0) le = launch_step_fused(a, g->maps[in], g->B, s);
+        if (tiles) {
+            use_tiles(g, a);
+            le = launch_step_tile(a, g->B, s);
+        } else if (g->kind == 0) le = launch_step_fused(a, g->maps[in], g->B, s);
         else if (g->kind == 1) le = launch_xsweep(a, g->B, s);
         else le = launch_ysweep(a, g->B, s);
         if (le != cudaSuccess) return set_err(CLIFFS_ERR_CUDA, "sweep launch: %s", cudaGetErrorString(le));
@@ -1444,17 +1509,25 @@ int cliffs_run_persistent(cliffs_grid* g, int64_t n) {
         CK(cudaGetDevice(&dev));
         CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         g->pblocks = sms * std::max(1, batch_blocks_per_sm(g->cfg.coords != 1));
+        g->pblocks_tile = sms * tile_blocks_per_sm(tile_max_rows());
     }
+    // no more blocks than the batch has work (each one more makes the barrier slower)
+    const bool tiles = by_tiles(g);
+    const long long work = (tiles ? (long long)g->tile.items.size() : ((long long)g->march.items.size() + fused_warps_per_block() - 1) /
+                                                                          fused_warps_per_block()) * g->B;
+    const int blocks = (int)std::min<long long>(tiles ? g->pblocks_tile : g->pblocks, work);
     // launch arguments; all padding zeroed so that they compare byte for byte
-    struct Key { StepArgs a; BatchArgs b; } k;
+    struct Key { StepArgs a; BatchArgs b; long long tiles; } k;
     std::memset(&k, 0, sizeof(k));
     fill_step_args(g, k.a, 0, 1);
     k.a.eta_out = nullptr;
-    fused_ring(last >= g->cfg.maxout, &k.a.nslots, &k.a.slot_floats);
+    if (tiles) use_tiles(g, k.a);
+    else fused_ring(last >= g->cfg.maxout, &k.a.nslots, &k.a.slot_floats);
+    k.tiles = tiles;
     k.a.eta_in = k.a.u_in = k.a.v_in = nullptr;
     k.a.limit = nullptr;
     if (g->inject_cycles > 0) {
-        // fault injection: every ring slot of this run waits for bytes that never come
+        // fault injection: the grid barrier of this run waits for an arrival that never comes
         k.a.wait_cycles = g->inject_cycles;
         k.a.tx_pad = 16;
         g->inject_cycles = 0;
@@ -1505,13 +1578,12 @@ int cliffs_run_persistent(cliffs_grid* g, int64_t n) {
         if (g->gexec) { cudaGraphExecDestroy(g->gexec); g->gexec = nullptr; }
         // the graph: copy the control block in from its pinned host image, then the
         // cooperative launch
-        StepMaps2 mm;
-        mm.m[0] = g->maps[0];
-        mm.m[1] = g->maps[1];
         cudaGraph_t graph = nullptr;
         CK(cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal));
         cudaError_t e1 = cudaMemcpyAsync(g->ctl_d, g->ctl_h, 4 * sizeof(long long), cudaMemcpyHostToDevice, g->cap);
-        cudaError_t e2 = e1 == cudaSuccess ? launch_batch(k.a, mm, b, g->pblocks, g->cap) : e1;
+        cudaError_t e2 = e1;
+        if (e2 == cudaSuccess)
+            e2 = tiles ? launch_batch_tile(k.a, b, blocks, g->cap) : launch_batch(k.a, StepMaps2{{g->maps[0], g->maps[1]}}, b, blocks, g->cap);
         cudaError_t e3 = cudaStreamEndCapture(g->cap, &graph);
         if (e2 != cudaSuccess || e3 != cudaSuccess) {
             if (graph) cudaGraphDestroy(graph);
@@ -1785,11 +1857,11 @@ static int adjoint_core(cliffs_grid* g, int scenario, int64_t n, int32_t checkpo
     // state `in` (fields fin floats apart, read through the descriptors M) to state `out`
     // (fields fout apart)
     auto step1 = [&](float* in, long long fin, const StepMaps& M, float* out, long long fout, long long j) -> int {
-        a.eta_in = in; a.u_in = in + fin; a.v_in = in + 2 * fin;
+        a.eta_in = in; a.u_in = in + fin; a.v_in = in + 2 * fin; a.fs_in = fin;
         a.eta_out = out; a.fs_out = fout;
         a.yfirst = g->cfg.alternate && ((s0 + j) & 1);     // the forward's parity: steps since set_initial
-        a.items = g->items_dev;
-        a.nitems = (int)g->items.size();
+        a.items = g->march.dev;
+        a.nitems = (int)g->march.items.size();
         if (g->bnd_any) {                                  // boundary input, as in cliffs_step_n
             const int rci = impose_boundary(g, in, in + fin, in + 2 * fin, g->t_start + (double)(s0 + j) * g->cfg.dt);
             if (rci) return rci;
@@ -2036,6 +2108,7 @@ int cliffs_set_rows_per_warp(cliffs_grid* g, int32_t rows) {
     if (!g->have_bathy) return set_err(CLIFFS_ERR_STATE, "set_bathy first (it chooses the geometry)");
     if (g->kind != 0) return set_err(CLIFFS_ERR_ARG, "a 1D grid has no tile shape");
     if (rows < 1 || rows > 8192) return set_err(CLIFFS_ERR_ARG, "rows per warp %d outside 1..8192", rows);
+    g->S_set = true;
     return set_rows_per_warp(g, rows);
 }
 
@@ -2083,8 +2156,8 @@ int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32
         if (S > 2 * g->ny && S != list[0]) break;
         rc = set_rows_per_warp(g, S);
         if (rc) break;
-        a.S = g->S; a.nseg = g->nseg; a.samp_ptr = g->samp_ptr; a.samp = g->samp;
-        a.items = g->items_dev; a.nitems = (int)g->items.size();
+        a.S = g->S; a.nseg = g->nseg; a.samp_ptr = g->march.samp_ptr; a.samp = g->march.samp;
+        a.items = g->march.dev; a.nitems = (int)g->march.items.size();
         float tbest = 1e30f;
         for (int t = 0; t <= trials; ++t) {             // the first launch warms up
             cudaMemsetAsync(flush, t & 0xff, flush_bytes, s);
@@ -2110,6 +2183,7 @@ int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32
     cudaMemcpy(h, g->err, sizeof(h), cudaMemcpyDeviceToHost);
     cudaMemset(g->err, 0, sizeof(h));
     const int rc2 = set_rows_per_warp(g, rc ? oldS : bestS);
+    g->S_set = !rc && !rc2;
     if (ncand) *ncand = n;
     if (rc) return rc;
     if (rc2) return rc2;

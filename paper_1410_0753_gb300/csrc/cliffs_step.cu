@@ -11,6 +11,8 @@
 //                the gauge / enclosed-grid sampling.
 //  k_batch       the same per-warp work in a persistent cooperative kernel that loops over
 //                the steps of a batch of scenarios, with a grid barrier between steps.
+//                (k_step_tile and k_batch_tile, tile_kernels.cuh: both by tiles, for grids
+//                that do not fill the GPU with marching warps.)
 //  k_xsweep      x-sweep alone (1D grids along x).
 //  k_ysweep      y-sweep alone (1D grids along y).
 // Variants (template parameters): spherical metric (SPH), friction on (FRIC), a y-first step

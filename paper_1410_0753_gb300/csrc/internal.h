@@ -25,6 +25,7 @@ struct SweepConst {
 // element (b, r, c) lives at b * plane + r * pitch + c.
 struct StepArgs {
     const float* eta_in; const float* u_in; const float* v_in;
+    long long fs_in;                 // floats from eta to u and from u to v of the input state
     float* eta_out;                  // u and v follow at the field stride
     long long fs_out;                // floats from eta to u and from u to v of the output state
     const float* d;                  // [ny][pitch], FP32 depth
@@ -50,6 +51,7 @@ struct StepArgs {
     const int4* items;               // fused kernel: per warp (strip, first row, end row)
     int nitems;
     int nslots, slot_floats;         // ring of a fused warp: slots and floats per slot
+    int tile_rows;                   // rows of the largest tile, halo included (k_step_tile, k_batch)
     int walls;                       // itopo = 0: nodes with d < dwall are walls
     SweepConst K;
     int sph;                         // geographic grid: x metric scaled per row
@@ -112,10 +114,9 @@ struct StepMaps2 {
     StepMaps m[2];                   // [k]: buffer k is the input
 };
 
-// The batched persistent run (k_batch). ctl lives in device memory so that one captured
+// The batched persistent run (k_batch, k_batch_tile). ctl lives in device memory so that one captured
 // graph serves every call: ctl[0] = steps done before the launch, ctl[1] = steps done after
-// it, ctl[2] = grid barrier (arrival count in the low 32 bits, generation in the high 32),
-// ctl[3] = work-item ticket counters for even (low 32 bits) and odd (high 32) steps.
+// it, ctl[2] = grid barrier (arrival count in the low 32 bits, generation in the high 32).
 // Interpolation of one step's boundary input per edge: record k and weight w toward k + 1.
 struct BndRow {
     long long k[4];
@@ -167,13 +168,18 @@ __device__ __forceinline__ void bnd_apply(float* eta, float* u, float* v, int pi
     eta[o] = (float)val[2];
 }
 
-// launchers (cliffs_step.cu)
+// launchers (cliffs_step.cu, cliffs_tile.cu)
+cudaError_t launch_step_fused(const StepArgs& a, const StepMaps& m, int batch, cudaStream_t s);
 cudaError_t launch_batch(const StepArgs& a, const StepMaps2& mm, const BatchArgs& b, int blocks, cudaStream_t s);
 int batch_blocks_per_sm(bool sph);
-cudaError_t launch_step_fused(const StepArgs& a, const StepMaps& m, int batch, cudaStream_t s);
 int fused_blocks_per_sm(bool sph);
 void fused_ring(bool maxwave, int* nslots, int* slot_floats);
 int fused_warps_per_block();
+cudaError_t launch_step_tile(const StepArgs& a, int batch, cudaStream_t s);
+cudaError_t launch_batch_tile(const StepArgs& a, const BatchArgs& b, int blocks, cudaStream_t s);
+int tile_warps_per_block();
+int tile_blocks_per_sm(int tile_rows);
+int tile_max_rows();             // the largest tile_rows of which two blocks fit on an SM
 cudaError_t launch_xsweep(const StepArgs& a, int batch, cudaStream_t s);
 cudaError_t launch_ysweep(const StepArgs& a, int batch, cudaStream_t s);
 

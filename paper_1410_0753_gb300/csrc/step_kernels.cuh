@@ -62,10 +62,17 @@ __device__ __forceinline__ void tma_box2(float* dst, const CUtensorMap* m, uint6
         : "memory");
 }
 
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* m) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
+}
 // A value that is the same in every lane, through an instruction whose result is uniform by
 // construction: the compiler then keeps what derives from it (row counters, ring positions)
 // in uniform registers and branches on it without convergence barriers.
 __device__ __forceinline__ int uniform(int x) { return __reduce_max_sync(FULL, x); }
+__device__ __forceinline__ long long uniform64(long long x) {
+    const unsigned lo = __reduce_max_sync(FULL, (unsigned)x), hi = __reduce_max_sync(FULL, (unsigned)(x >> 32));
+    return (long long)(((unsigned long long)hi << 32) | lo);
+}
 
 // ------------------------------------------------------------------ epilogue
 // Nodes (r, c) and (r, c+1) of the step input, for the kernels without TMA; nodes outside
@@ -174,7 +181,7 @@ __device__ __forceinline__ void write_samples(const StepArgs& a, const StepOut& 
         float* out = it.z == 0 ? rg : O.rec_n;
         if (!out) continue;
         const float* q = st + ((long long)it.x * a.pitch + it.y);
-        const float e = q[0], u = q[a.fs_out], v = q[2 * a.fs_out];
+        const float e = __ldcg(q), u = __ldcg(q + a.fs_out), v = __ldcg(q + 2 * a.fs_out);
         out[3 * it.w + 0] = e;
         out[3 * it.w + 1] = u;
         out[3 * it.w + 2] = v;
@@ -498,19 +505,15 @@ struct FusedWarp {
         }
     }
 
-    // Process work item `idx` (strip, rows) of scenario b_ for the step described by O_.
-    // Returns false when a wait expired (the warp's copies have landed when it returns).
-    __device__ __forceinline__ bool run_item(int idx, int b_, const StepOut& O_) {
-        O = O_;
-        b = uniform(b_);
+    // Take work item `idx` (strip, rows): what does not depend on the state.
+    __device__ __forceinline__ void take_item(int idx) {
         const int4 item = __ldg(a.items + idx);          // (strip, first row, end row)
-        c0 = uniform(item.x) * XOUT;                          // window columns c0 .. c0 + 63 (fused_strips)
+        c0 = uniform(item.x) * XOUT;                     // window columns c0 .. c0 + 63 (fused_strips)
         const int cA = c0 + 2 * lane;
         r0 = uniform(item.y);
         r1 = uniform(item.z);
         k0 = r0 - 3;
         kpast = min(r1, a.ny - 1);
-        tx = (O.emax ? 6u : 4u) * ARR_FLOATS * 4u + a.tx_pad;
         colA = cA < a.nx;
         colB = cA + 1 < a.nx;
         // the output columns: c0 + 4 .. c0 + 59, and from the domain's first column in the
@@ -522,16 +525,24 @@ struct FusedWarp {
         wallx = c0 == 0 || c0 + XWIN >= a.nx;
         walls = wall_ends_x(cA, a.nx);
         ends = OPEN ? open_ends_x(a, cA) : 0u;
+        float2 hr = v2(0.f), k2 = v2(0.f);
+        if (colA) { hr.x = __ldg(a.xb + cA); k2.x = __ldg(a.xk + cA); }
+        if (colB) { hr.y = __ldg(a.xb + cA + 1); k2.y = __ldg(a.xk + cA + 1); }
+        m0 = XMet2{v2(0.f), hr, k2};
+    }
+
+    // Process the item taken (number idx) of scenario b_ for the step described by O_. Returns
+    // false when a wait expired (the warp's copies have landed when it returns).
+    __device__ __forceinline__ bool run_item(int idx, int b_, const StepOut& O_) {
+        O = O_;
+        b = b_;
+        tx = (O.emax ? 6u : 4u) * ARR_FLOATS * 4u + a.tx_pad;
         // the slots the open-water march reads (with max-wave due its rows count too)
         ntot = ((O.emax ? r1 + 1 : kpast) - k0) / SLOT_ROWS + 1;
         nfill = nread = 0;
         cs = head;
         const int first = head;
         while (nfill < min(a.nslots, ntot)) fill();
-        float2 hr = v2(0.f), k2 = v2(0.f);
-        if (colA) { hr.x = __ldg(a.xb + cA); k2.x = __ldg(a.xk + cA); }
-        if (colB) { hr.y = __ldg(a.xb + cA + 1); k2.y = __ldg(a.xk + cA + 1); }
-        m0 = XMet2{v2(0.f), hr, k2};
         ym.init();
         // An open first or last row and eq. (solver1)'s flux around one take the general path: no
         // open water from row kgen on, and no start in open water above row 0.
@@ -602,11 +613,17 @@ k_step_fused(const __grid_constant__ StepMaps M, const __grid_constant__ StepArg
     const int gw = uniform(blockIdx.x * FUSED_WARPS + wib);
     const int b = blockIdx.y;
     if (gw >= a.nitems) return;
+    FusedWarp<SPH, FRIC, YF, S1, OPEN> W(a);
+    W.setup(smem_raw, wib);
+    W.take_item(gw);
+    if (W.lane == 0) {
+        prefetch_map(&M.s);
+        prefetch_map(&M.d);
+        if (a.emax) prefetch_map(&M.mw);
+    }
     if (a.limit && __all_sync(FULL, a.step > a.limit[b])) return;
     // a wait of an earlier launch expired: do not start new copies
     if (__any_sync(FULL, *reinterpret_cast<volatile int*>(a.err) & ERRF_TIMEOUT)) return;
-    FusedWarp<SPH, FRIC, YF, S1, OPEN> W(a);
-    W.setup(smem_raw, wib);
     W.run_item(gw, b, step_out(&M, a));
     W.report();
 }
@@ -615,7 +632,8 @@ k_step_fused(const __grid_constant__ StepMaps M, const __grid_constant__ StepArg
 // Grid-wide barrier of a cooperative launch. Thread 0 of every block adds one arrival to the
 // low half of *bar; the last arrival clears the count and advances the generation in the high
 // half, which the others wait on for at most `limit` cycles before setting the timeout flag.
-// Returns false when the run must stop (a wait expired here or anywhere else).
+// Returns false when the run must stop (a wait expired here or, as of the arrival, anywhere
+// else: the flag is read while waiting, so it costs no latency of its own).
 __device__ __forceinline__ bool grid_sync(unsigned long long* bar, unsigned nblocks, long long limit, int* err) {
     __shared__ int go;
     asm volatile("fence.proxy.async.global;" ::: "memory");    // outputs before the next TMA reads
@@ -624,6 +642,7 @@ __device__ __forceinline__ bool grid_sync(unsigned long long* bar, unsigned nblo
         int ok = 1;
         __threadfence();
         const unsigned long long old = atomicAdd(bar, 1ull);
+        const int flag = *reinterpret_cast<volatile int*>(err);
         const unsigned gen = (unsigned)(old >> 32);
         if ((unsigned)old == nblocks - 1) {
             // last arrival: count back to zero and generation + 1, in one atomic
@@ -631,28 +650,26 @@ __device__ __forceinline__ bool grid_sync(unsigned long long* bar, unsigned nblo
         } else {
             volatile unsigned* vgen = reinterpret_cast<volatile unsigned*>(bar) + 1;
             const long long t0 = clock64();
-            while (*vgen == gen) {
+            while (*vgen == gen)
                 if (clock64() - t0 > limit) { ok = 0; break; }
-                __nanosleep(32);
-            }
         }
         __threadfence();
         if (!ok) atomicOr(err, ERRF_TIMEOUT);
-        go = ok && !(*reinterpret_cast<volatile int*>(err) & ERRF_TIMEOUT);
+        go = ok && !(flag & ERRF_TIMEOUT);
     }
     __syncthreads();
     asm volatile("fence.proxy.async.global;" ::: "memory");
-    return go;
+    return __all_sync(FULL, go);
 }
 
 // Steps ctl[0]+1 .. ctl[1] of a batch of scenarios in one launch. Scenarios are taken in
 // decreasing order of duration, so those still running at a step are the first nact[step]
-// of `order`; the step's (scenario, item) pairs are numbered scenario-major and each warp
-// takes the next number from a ticket counter until none are left, then the warps meet at
-// the grid barrier before the next step reads what this one wrote. Two ticket counters
-// (the halves of ctl[3]) alternate by step parity; block 0 clears the one the next step
-// uses while the other is in use. A scenario that has stopped keeps its last state in the
-// buffer of its last step's parity.
+// of `order`; the step's (scenario, item) pairs are numbered scenario-major and warp w of W
+// takes numbers w, w + W, .. (items cost the same, see cut_items; handing them out by an
+// atomic counter put a round trip to L2 before every item, and on small grids queued every
+// warp at one address), then the warps meet at the grid barrier before the next step reads
+// what this one wrote. A scenario that has stopped keeps its last state in the buffer of its
+// last step's parity.
 // With ALT (the alternating order) the odd-indexed steps (st - 1 odd) sweep y first: a second
 // per-warp worker of the y-first kind shares the warp's ring, barriers and ring position.
 template <bool SPH, bool FRIC, bool S1, bool OPEN, bool ALT>
@@ -660,9 +677,10 @@ __global__ void __launch_bounds__(FUSED_WARPS * 32, 4)
 k_batch(const __grid_constant__ StepMaps2 MM, const __grid_constant__ StepArgs a, const __grid_constant__ BatchArgs B) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int wib = threadIdx.x >> 5;
-    const long long step0 = B.ctl[0], step_end = B.ctl[1];
-    unsigned* tickets = reinterpret_cast<unsigned*>(B.ctl + 3);
-    if (*reinterpret_cast<volatile int*>(a.err) & ERRF_TIMEOUT) return;
+    const unsigned gw = (unsigned)uniform(blockIdx.x * FUSED_WARPS + wib), nw = gridDim.x * FUSED_WARPS;
+    const long long step0 = uniform64(B.ctl[0]), step_end = uniform64(B.ctl[1]);
+    if (__any_sync(FULL, *reinterpret_cast<volatile int*>(a.err) & ERRF_TIMEOUT)) return;
+    int taken = -1;                                // the item taken last
     FusedWarp<SPH, FRIC, false, S1, OPEN> W(a);
     W.setup(smem_raw, wib);
     FusedWarp<SPH, FRIC, true, S1, OPEN> WY(a);
@@ -693,16 +711,16 @@ k_batch(const __grid_constant__ StepMaps2 MM, const __grid_constant__ StepArgs a
         StepOut O{odd ? &MM.m[0] : &MM.m[1], odd ? B.eta[1] : B.eta[0], mx ? B.emax : nullptr,
                   (B.grec && st % B.gout == 0) ? B.grec + (st / B.gout) * B.grec_row : nullptr,
                   (B.nrec && st % B.bndout == 0) ? B.nrec + (st / B.bndout) * B.nrec_row : nullptr};
-        const int na = B.nact ? (st < B.nact_len ? __ldg(B.nact + st) : 0) : B.nall;
+        const int na = B.nact ? (st < B.nact_len ? uniform(__ldg(B.nact + st)) : 0) : B.nall;
         const unsigned total = (unsigned)na * (unsigned)a.nitems;
-        if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(tickets + (odd ? 0 : 1), 0u);
         bool ok = true;
-        while (ok) {
-            unsigned t = 0;
-            if (W.lane == 0) t = atomicAdd(tickets + (odd ? 1 : 0), 1u);
-            t = (unsigned)uniform((int)__shfl_sync(FULL, t, 0));
-            if (t >= total) break;
+        for (unsigned t = gw; ok && t < total; t += nw) {
             const int item = (int)(t % (unsigned)a.nitems), scen = uniform(__ldg(B.order + t / (unsigned)a.nitems));
+            if (ALT || item != taken) {
+                if (yf) WY.take_item(item);
+                else W.take_item(item);
+                taken = item;
+            }
             ok = yf ? WY.run_item(item, scen, O) : W.run_item(item, scen, O);
         }
         if (yf) { W.head = WY.head; W.phase = WY.phase; }

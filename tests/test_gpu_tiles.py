@@ -1,0 +1,72 @@
+"""The step by tiles (k_step_tile, k_batch_tile) against the marching warps it stands in for.
+Both run the same arithmetic per node, so the results are equal bit for bit: state, max-wave and gauge records. Sizes at the edges of windows (64
+columns, 56 finished) and tiles, one row or column either side, down to the smallest grids.
+"""
+import numpy as np
+import pytest
+
+from paper_1410_0753_gb300 import CliffsGrid
+
+pytestmark = pytest.mark.gpu
+
+
+def _grid(nx, ny, seed=3, coords=1, **kw):
+    """A shelf with a shore, an island and a hump whose wave floods and dries nodes."""
+    rng = np.random.default_rng(seed)
+    X, Y = np.meshgrid((np.arange(nx) + 0.5) / nx, (np.arange(ny) + 0.5) / ny)
+    d = 30.0 * (1.0 - 1.15 * X) + 4.0 * np.sin(7 * X + 5 * Y) + rng.normal(0, 0.3, (ny, nx))
+    d -= 60.0 * np.exp(-((X - 0.4) ** 2 + (Y - 0.55) ** 2) / 0.01)
+    d = np.round(d * 64) / 64
+    if coords == 1:
+        x, y, ds = 50.0 * np.arange(nx), 40.0 * np.arange(ny), 40.0
+    else:
+        x, y, ds = 10.0 + np.arange(nx) / 600.0, 40.0 + np.arange(ny) / 600.0, 120.0
+    gauges = [(nx // 2, ny // 2), (0, 0), (nx - 1, ny - 1), (min(nx - 1, 59), ny // 3)]
+    g = CliffsGrid(nx, ny, 0.6 * ds / np.sqrt(9.81 * 45.0), coords=coords, manning_n2=kw.pop("manning_n2", 6e-4),
+                   gauges=gauges, maxout=3, gout=2, **kw)
+    g.set_bathy(x, y, d, True)
+    eta = 1.5 * np.exp(-((X - 0.65) ** 2 + (Y - 0.5) ** 2) / 0.02)
+    return g, np.where(d > 0, eta, 0.0).astype(np.float32)
+
+
+def _result(g, b=0):
+    return [*g.state(b), *g.maxwave(b), g.gauges(b)]
+
+
+def _same(a, b):
+    for p, q in zip(a, b):
+        assert np.array_equal(p, q)
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(coords=0), dict(alternate=1, open_edges=9), dict(solver=1, open_edges=6),
+                                dict(itopo=0, dwall=2.0), dict(manning_n2=0.0, transverse=0)])
+@pytest.mark.parametrize("nx,ny", [(3, 3), (64, 9), (65, 40), (57, 83), (119, 6), (120, 97), (121, 16), (300, 161)])
+def test_tiles_equal_marching_warps(nx, ny, kw):
+    outs = []
+    for how in ("tiles", "march", "persistent", "march persistent"):
+        g, eta = _grid(nx, ny, **kw)
+        if "march" in how:
+            g.set_rows_per_warp(7)                   # a tile shape of the caller's: marching warps
+        g.set_initial(eta)
+        g.step(17, persistent="persistent" in how)
+        outs.append(_result(g))
+        g.close()
+    assert np.isfinite(outs[0][0]).all()
+    for o in outs[1:]:
+        _same(outs[0], o)
+
+
+def test_batch_with_durations_by_tiles_equals_marching_warps():
+    durations = np.array([11, 4, 0, 17, 9], np.int64)
+    outs = []
+    for march, persistent in ((0, 0), (1, 0), (0, 1), (1, 1)):
+        g, eta = _grid(130, 70, batch=5)
+        if march:
+            g.set_rows_per_warp(12)
+        g.set_initial(np.stack([eta * (0.3 + 0.2 * b) for b in range(5)]))
+        g.set_durations(durations)
+        g.step(17, persistent=bool(persistent))
+        outs.append([r for b in range(5) for r in _result(g, b)])
+        g.close()
+    for o in outs[1:]:
+        _same(outs[0], o)

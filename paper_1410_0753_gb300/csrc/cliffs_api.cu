@@ -1422,6 +1422,28 @@ int cliffs_step_n(cliffs_grid* g, int64_t n) {
     StepArgs a;
     const bool tiles = by_tiles(g) && g->inject_cycles <= 0;
     const double t_end = g->bnd_any ? bnd_end(g) : 1e300;
+    // 1D lines: all the steps in one launch (at most LINE_STEPS, some tens of milliseconds),
+    // except one step alone, lines too long for a block, boundary input, timed launches and the
+    // spherical source term of a line along y
+    const long long LINE_STEPS = 65536;
+    if (g->kind != 0 && n > 1 && !g->timing && !g->bnd_any && line_fits(g->kind == 1 ? g->nx : g->ny) &&
+        !(g->kind == 2 && g->cfg.coords != 1)) {
+        BatchArgs b{};
+        for (int i = 0; i < 2; ++i) b.eta[i] = g->eta[i];
+        b.emax = g->emax;
+        b.maxout = g->cfg.maxout;
+        b.gout = g->cfg.gout;
+        b.grec = g->G ? g->grec : nullptr;
+        b.grec_row = (long long)g->G * 3;
+        fill_step_args(g, a, 0, 1);
+        a.samp = g->items_d;
+        for (; n > 0; n -= std::min(n, (int64_t)LINE_STEPS)) {
+            const long long m = std::min((long long)n, LINE_STEPS);
+            const cudaError_t le = launch_line(a, b, g->B, g->step, m, (int)g->samples.size(), g->kind == 2, s);
+            if (le != cudaSuccess) return set_err(CLIFFS_ERR_CUDA, "line launch: %s", cudaGetErrorString(le));
+            g->step += m;
+        }
+    }
     for (long long k = 0; k < n; ++k) {
         const long long st = g->step + 1;
         const int in = (int)(g->step & 1), out = 1 - in;

@@ -180,6 +180,10 @@ cudaError_t launch_batch_tile(const StepArgs& a, const BatchArgs& b, int blocks,
 int tile_warps_per_block();
 int tile_blocks_per_sm(int tile_rows);
 int tile_max_rows();             // the largest tile_rows of which two blocks fit on an SM
+bool line_fits(int nodes);        // a 1D line of this many nodes fits in one block (cliffs_line.cu)
+// steps step0 + 1 .. step0 + n of a 1D grid's scenarios, the samples in a.samp
+cudaError_t launch_line(const StepArgs& a, const BatchArgs& b, int batch, long long step0, long long n, int nsamp,
+                        int along_y, cudaStream_t s);
 cudaError_t launch_xsweep(const StepArgs& a, int batch, cudaStream_t s);
 cudaError_t launch_ysweep(const StepArgs& a, int batch, cudaStream_t s);
 

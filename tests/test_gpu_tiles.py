@@ -1,5 +1,6 @@
-"""The step by tiles (k_step_tile, k_batch_tile) against the marching warps it stands in for.
-Both run the same arithmetic per node, so the results are equal bit for bit: state, max-wave and gauge records. Sizes at the edges of windows (64
+"""The step by tiles (k_step_tile, k_batch_tile) and the one-launch 1D run (k_line) against the
+launches they stand in for. All of them run the same arithmetic per node, so the results are
+equal bit for bit: state, max-wave and gauge records. Sizes at the edges of windows (64
 columns, 56 finished) and tiles, one row or column either side, down to the smallest grids.
 """
 import numpy as np
@@ -70,3 +71,19 @@ def test_batch_with_durations_by_tiles_equals_marching_warps():
         g.close()
     for o in outs[1:]:
         _same(outs[0], o)
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(open_edges=1), dict(open_edges=10), dict(solver=1), dict(manning_n2=0.0)])
+@pytest.mark.parametrize("n", [3, 4, 55, 56, 57, 61, 113, 613, 1900])
+@pytest.mark.parametrize("along_y", [0, 1])
+def test_line_in_one_launch_equals_a_launch_per_step(n, along_y, kw):
+    outs = []
+    for per in (1, 23):
+        g, eta = _grid(1, n, **kw) if along_y else _grid(n, 1, **kw)
+        g.set_initial(eta, 0.2 * eta, 0.1 * eta)
+        for _ in range(23 // per):
+            g.step(per)                              # one step alone takes the kernel per step
+        outs.append(_result(g))
+        g.close()
+    assert np.isfinite(outs[0][0]).all()
+    _same(outs[0], outs[1])

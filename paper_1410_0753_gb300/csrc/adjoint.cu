@@ -37,7 +37,7 @@ constexpr int TP = ALINES + 1;              // shared tile pitch (no bank confli
 
 struct ANode { float e, w, t, d, c; };      // post-(b) state of a node or of a mirror ghost
 struct ABar { float e, w, t; };             // adjoints of (eta, w, t)
-struct AMet { float il, ir, k2, sdt; };     // 1/ds_left, 1/ds_right, dt^2/(ds_l+ds_r), dt tan/R
+struct AMet { float hl, hr, k2, nsdt; };    // 1/(2 ds_left), 1/(2 ds_right), dt^2/(ds_l+ds_r), -dt tan/R
 
 // Interface between a left node b and a right node a (times the interval): the fluxes of
 // p, q (eq. (eqQ)) and t (eq. (pq3)) and the differences their derivatives need.
@@ -82,7 +82,7 @@ template <bool SRC, bool S1>
 __device__ __forceinline__ void a_dstage(const ANode& L, const ANode& C, const ANode& R, const AMet& m,
                                          const SweepConst& K, float& e2, float& w2) {
     const AIface fl = a_iface(L, C), fr = a_iface(C, R);
-    const float QpL = fl.qp * m.il, QpR = fr.qp * m.ir, QqL = fl.qq * m.il, QqR = fr.qq * m.ir;
+    const float QpL = fl.qp * (2.f * m.hl), QpR = fr.qp * (2.f * m.hr), QqL = fl.qq * (2.f * m.hl), QqR = fr.qq * (2.f * m.hr);
     const float hdt = K.half_dt;
     float dp, dq;
     if (S1) {
@@ -98,7 +98,7 @@ __device__ __forceinline__ void a_dstage(const ANode& L, const ANode& C, const A
     dp -= F.adt;
     dq -= F.adt;
     if (SRC) {
-        const float s = m.sdt * C.c * C.w;
+        const float s = (-m.nsdt) * C.c * C.w;
         dp += s;
         dq -= s;
     }
@@ -114,8 +114,8 @@ __device__ __forceinline__ void a_dstage_adj(const ANode& L, const ANode& C, con
                                              const SweepConst& K, float ge, float gw, float gt,
                                              ABar& bL, ABar& bC, ABar& bR) {
     const AIface fl = a_iface(L, C), fr = a_iface(C, R);
-    const float QpL = fl.qp * m.il, QpR = fr.qp * m.ir, QqL = fl.qq * m.il, QqR = fr.qq * m.ir;
-    const float QtL = fl.qt * m.il, QtR = fr.qt * m.ir;
+    const float QpL = fl.qp * (2.f * m.hl), QpR = fr.qp * (2.f * m.hr), QqL = fl.qq * (2.f * m.hl), QqR = fr.qq * (2.f * m.hr);
+    const float QtL = fl.qt * (2.f * m.hl), QtR = fr.qt * (2.f * m.hr);
     const float hdt = K.half_dt;
     const float lp = C.w + C.c, lq = C.w - C.c;
     AIface flr{};
@@ -134,7 +134,7 @@ __device__ __forceinline__ void a_dstage_adj(const ANode& L, const ANode& C, con
     dp -= F.adt;
     dq -= F.adt;
     if (SRC) {
-        const float s = m.sdt * C.c * C.w;
+        const float s = (-m.nsdt) * C.c * C.w;
         dp += s;
         dq -= s;
     }
@@ -170,14 +170,14 @@ __device__ __forceinline__ void a_dstage_adj(const ANode& L, const ANode& C, con
         eC += G * C.w * (-4.f / 3.f) * rcp_approx(C.e + C.d);
     }
     if (SRC) {
-        const float gs = (gdp - gdq) * m.sdt;
+        const float gs = (gdp - gdq) * (-m.nsdt);
         cC += gs * C.w;
         wC += gs * C.c;
     }
     // Q(a, b) ds = 1/2 (lam_a + lam_b)(r_a - r_b) - g (d_a - d_b): partials with respect to
     // w and c of both sides, for p (lam = w + c, r = w + 2c) and q (lam = w - c, r = w - 2c)
     {   // left interface: b = L, a = C
-        const float A = gQpL * m.il, B = gQqL * m.il, T = gQtL * m.il;
+        const float A = gQpL * (2.f * m.hl), B = gQqL * (2.f * m.hl), T = gQtL * (2.f * m.hl);
         const float hp = 0.5f * fl.dw + fl.dcs, hq = 0.5f * fl.dw - fl.dcs;
         const float sp = fl.sw + fl.S, sq = fl.sw - fl.S;
         wC += A * (hp + 0.5f * sp) + B * (hq + 0.5f * sq) + T * 0.5f * fl.dtt;
@@ -188,7 +188,7 @@ __device__ __forceinline__ void a_dstage_adj(const ANode& L, const ANode& C, con
         bL.t -= T * 0.5f * fl.sw;
     }
     {   // right interface: b = C, a = R
-        const float A = gQpR * m.ir, B = gQqR * m.ir, T = gQtR * m.ir;
+        const float A = gQpR * (2.f * m.hr), B = gQqR * (2.f * m.hr), T = gQtR * (2.f * m.hr);
         const float hp = 0.5f * fr.dw + fr.dcs, hq = 0.5f * fr.dw - fr.dcs;
         const float sp = fr.sw + fr.S, sq = fr.sw - fr.S;
         bR.w += A * (hp + 0.5f * sp) + B * (hq + 0.5f * sq) + T * 0.5f * fr.dtt;
@@ -238,133 +238,104 @@ __device__ __forceinline__ void a_open_ghost_adj(const ANode& C, const ANode& Gh
 }
 
 // ------------------------------------------------------------------ packed open water
-// The same adjoint of (d) for the two nodes of a lane at once (packed FP32x2), for windows
-// where every node is wet: real neighbours, no ghosts.
-__device__ __forceinline__ float2 rcp2(float2 x) { return make_float2(rcp_approx(x.x), rcp_approx(x.y)); }
-
-struct N2 { float2 e, w, t, d, c; };
-struct AIface2 { float2 dw, dcs, sw, S, dtt, qp, qq, qt; };
-
-__device__ __forceinline__ AIface2 a_iface2(const N2& b, const N2& a) {
-    AIface2 f;
-    const float2 de = sub2(a.e, b.e);
-    f.S = add2(a.c, b.c);
-    f.dcs = mul2(mul2(v2(GRAV), add2(de, sub2(a.d, b.d))), rcp2(f.S));
-    f.dw = sub2(a.w, b.w);
-    f.sw = add2(a.w, b.w);
-    f.dtt = sub2(a.t, b.t);
-    const float2 y = mul2(f.sw, f.dcs), z = mul2(v2(GRAV), de), hdw = mul2(v2(0.5f), f.dw);
-    f.qp = fma2(hdw, add2(f.sw, f.S), add2(z, y));
-    f.qq = fma2(hdw, sub2(f.sw, f.S), sub2(z, y));
-    f.qt = mul2(mul2(v2(0.5f), f.sw), f.dtt);
-    return f;
-}
-
-// friction part of the adjoint for one node (adt = w k, see a_friction)
-__device__ __forceinline__ void fric_adj1(float gadt, float w, float t, float e, float d, float s2, float k,
-                                          bool clamped, float& wC, float& tC, float& eC) {
-    if (clamped) {
-        wC += gadt;
-    } else if (s2 > 1e-30f) {                      // below, k < 1e-15: no friction to speak of
-        const float G = gadt * k, rs2 = rcp_approx(s2);
-        wC += G * (1.f + w * w * rs2);
-        tC += G * w * t * rs2;
-        eC += G * w * (-4.f / 3.f) * rcp_approx(e + d);
-    }
-}
-
+// Adjoint of one sweep of a window whose nodes inside the line are all wet (no (b), no (e),
+// walls only at the line's ends), for the two nodes of a lane at once (packed FP32x2), on
+// the forward's form of the sweep: fluxes a, b, t of an interface and
+//   D = fl La + fr Ra + ck (Lb - Rb) + w kf,   w2 = w - D,
+//   N = fl Lb + fr Rb + ck (La - Ra) - sdt c w, e2 = e + N (N - 4c)/(4g),
+//   T = fl Lt + fr Rt,                          t2 = t - T,
+// with ck = c k2, fl, fr = dt/2 +- w k2 and kf the friction factor. Every node's adjoint goes to
+// its two fluxes, the two adjoints of a flux are added, and the interface is transposed
+// once (b's differences and sums give both sides' parts), about 100 packed operations where the transposed
+// stencil of each node by itself, on p and q, took 250.
+// wl: this lane's A is the line's first node; wr: the line's last node is its A (1) or B (2);
+// inA, inB: the interface on the right of A (of B) lies inside the line. edge: some lane of the
+// window has one of these.
 template <bool SRC>
-__device__ __forceinline__ void a_dstage_adj2(const N2& L, const N2& C, const N2& R, float2 il, float2 ir,
-                                              float2 k2, float2 sdt, const SweepConst& K, float2 ge, float2 gw,
-                                              float2 gt, float2 (&bL)[3], float2 (&bC)[3], float2 (&bR)[3]) {
-    const AIface2 fl = a_iface2(L, C), fr = a_iface2(C, R);
-    const float2 QpL = mul2(fl.qp, il), QpR = mul2(fr.qp, ir), QqL = mul2(fl.qq, il), QqR = mul2(fr.qq, ir);
-    const float2 QtL = mul2(fl.qt, il), QtR = mul2(fr.qt, ir);
-    const float2 nh = v2(-K.half_dt);
-    const float2 lp = add2(C.w, C.c), lq = sub2(C.w, C.c);
-    const float2 dQp = sub2(QpR, QpL), dQq = sub2(QqR, QqL);
-    float2 dp = fma2(mul2(lp, k2), dQp, mul2(nh, add2(QpL, QpR)));
-    float2 dq = fma2(mul2(lq, k2), dQq, mul2(nh, add2(QqL, QqR)));
-    float2 s2 = v2(0.f), kf = v2(0.f);
-    bool clA = false, clB = false;
-    const bool fric = K.fric != 0;
-    if (fric) {
-        float2 ex;
-        kf = fric_k2(C.w, C.t, C.c, K, s2, ex);
-        clA = ex.x >= 0.f;
-        clB = ex.y >= 0.f;
-        const float2 adt = mul2(C.w, kf);
-        dp = sub2(dp, adt);
-        dq = sub2(dq, adt);
+__device__ __forceinline__ void line_adjoint_open(float2 e, float2 w, float2 t, float2 d, float2 ge, float2 gw, float2 gt,
+                                                  float2 hl, float2 hr, float2 k2, float2 nsdt, const SweepConst& K,
+                                                  bool edge, bool wl, int wr, bool inA, bool inB, float2& oe,
+                                                  float2& ow, float2& ot) {
+    const float2 gh = mul2(v2(GRAV), add2(e, d));
+    const float2 rc = make_float2(rsqrt_approx(gh.x), rsqrt_approx(gh.y));     // 1/c
+    const float2 c = wave_speed2(add2(e, d));
+    auto dn = [](float x) { return __shfl_down_sync(FULL, x, 1); };
+    auto up = [](float x) { return __shfl_up_sync(FULL, x, 1); };
+    // the right interfaces, one by one as in the forward (iface_right)
+    auto dif = [](float2 p, float r) { return make_float2(__fsub_rn(p.y, p.x), __fsub_rn(r, p.y)); };
+    auto sum = [](float2 p, float r) { return make_float2(__fadd_rn(p.y, p.x), __fadd_rn(r, p.y)); };
+    const float wR = dn(w.x), cR = dn(c.x);
+    const float2 de = dif(e, dn(e.x)), dt = dif(t, dn(t.x)), dd = dif(d, dn(d.x));
+    const float2 dw = dif(w, wR), sw = sum(w, wR), sc = sum(c, cR);
+    const float2 z = mul2(v2(2.f * GRAV), de);
+    const float2 rs = make_float2(rcp_approx(sc.x), rcp_approx(sc.y));
+    const float2 dc = mul2(fma2(v2(2.f * GRAV), dd, z), rs);
+    float2 Ra = mul2(fma2(dw, sw, z), hr), Rb = mul2(fma2(dw, sc, mul2(sw, dc)), hr), Rt = mul2(mul2(sw, dt), hr);
+    float2 La = make_float2(up(Ra.y), Ra.x), Lb = make_float2(up(Rb.y), Rb.x), Lt = make_float2(up(Rt.y), Rt.x);
+    if (edge) {
+        if (wl) ghost_left(w.x, c.x, hl.x, La.x, Lb.x, Lt.x);
+        if (wr == 1) ghost_right(w.x, c.x, hr.x, Ra.x, Rb.x, Rt.x);
+        if (wr == 2) ghost_right(w.y, c.y, hr.y, Ra.y, Rb.y, Rt.y);
+    }
+    const float2 wk = mul2(w, k2), ck = mul2(c, k2);
+    const float2 fl = add2(K.hdt, wk), fr = sub2(K.hdt, wk);
+    const float2 da = sub2(La, Ra), db = sub2(Lb, Rb);
+    float2 N = fma2(ck, da, fma2(Rb, fr, mul2(Lb, fl)));
+    if (SRC) N = fma2(mul2(nsdt, c), w, N);
+    // node: to its fluxes, w and c
+    const float2 gh2 = mul2(ge, v2(0.5f * INV_GRAV));
+    const float2 gD = mul2(gw, v2(-1.f)), gT = mul2(gt, K.ntr);
+    const float2 gN = mul2(gh2, fma2(v2(-2.f), c, N));
+    float2 eC = ge, tC = gt;
+    float2 wC = fma2(fma2(gD, da, fma2(gN, db, mul2(gT, sub2(Lt, Rt)))), k2, gw);
+    float2 cC = fma2(fma2(gD, db, mul2(gN, da)), k2, mul2(mul2(gh2, v2(-2.f)), N));
+    if (K.fric) {
+        // adt = w k enters D: k ~ sqrt(s2) h^(-4/3), so dk/dw = k w / s2, dk/dt = k t / s2,
+        // dk/dh = -4/3 k / h (1/h = g / c^2); clamped, k = 1 is a constant
+        float2 s2, ex;
+        const float2 G = mul2(gD, fric_k2(w, t, c, K, s2, ex));
+        float2 u = make_float2(s2.x > 1e-30f ? rcp_approx(s2.x) : 0.f, s2.y > 1e-30f ? rcp_approx(s2.y) : 0.f);
+        float2 x = mul2(mul2(rc, rc), v2(-4.f / 3.f * GRAV));
+        if (ex.x >= 0.f) u.x = x.x = 0.f;
+        if (ex.y >= 0.f) u.y = x.y = 0.f;
+        const float2 Gw = mul2(G, w), Gu = mul2(Gw, u);
+        wC = fma2(Gu, w, add2(wC, G));
+        tC = fma2(Gu, t, tC);
+        eC = fma2(Gw, x, eC);
     }
     if (SRC) {
-        const float2 sw_ = mul2(mul2(sdt, C.c), C.w);
-        dp = add2(dp, sw_);
-        dq = sub2(dq, sw_);
+        const float2 gs = mul2(gN, nsdt);
+        cC = fma2(gs, w, cC);
+        wC = fma2(gs, c, wC);
     }
-    const float2 dcn = mul2(v2(0.25f), sub2(dp, dq));
-    // reverse sweep
-    float2 eC = ge, wC = gw, tC = gt;
-    float2 cC = mul2(ge, mul2(v2(2.f * INV_GRAV), dcn));
-    const float2 gdcn = mul2(ge, mul2(v2(2.f * INV_GRAV), add2(C.c, dcn)));
-    const float2 gdp = fma2(v2(0.5f), gw, mul2(v2(0.25f), gdcn));
-    const float2 gdq = fma2(v2(0.5f), gw, mul2(v2(-0.25f), gdcn));
-    float2 gQtL = v2(0.f), gQtR = v2(0.f);
-    if (K.transverse) {
-        const float2 wk = mul2(C.w, k2);
-        gQtL = mul2(gt, sub2(nh, wk));
-        gQtR = mul2(gt, add2(nh, wk));
-        wC = fma2(mul2(gt, k2), sub2(QtR, QtL), wC);
+    const float2 nck = mul2(gN, ck), dck = mul2(gD, ck);
+    float2 gLa = fma2(gD, fl, nck), gRa = sub2(mul2(gD, fr), nck);
+    float2 gLb = fma2(gN, fl, dck), gRb = sub2(mul2(gN, fr), dck);
+    const float2 gLt = mul2(gT, fl), gRt = mul2(gT, fr);
+    if (edge) {                                        // b = +-4 w c hl (hr) at the walls
+        if (wl) { const float x = 4.f * hl.x * gLb.x; wC.x += x * c.x; cC.x += x * w.x; }
+        if (wr == 1) { const float x = 4.f * hr.x * gRb.x; wC.x -= x * c.x; cC.x -= x * w.x; }
+        if (wr == 2) { const float x = 4.f * hr.y * gRb.y; wC.y -= x * c.y; cC.y -= x * w.y; }
     }
-    const float2 lpk = mul2(lp, k2), lqk = mul2(lq, k2);
-    const float2 gQpL = mul2(gdp, sub2(nh, lpk)), gQpR = mul2(gdp, add2(nh, lpk));
-    const float2 gQqL = mul2(gdq, sub2(nh, lqk)), gQqR = mul2(gdq, add2(nh, lqk));
-    const float2 glp = mul2(mul2(gdp, k2), dQp), glq = mul2(mul2(gdq, k2), dQq);
-    wC = add2(wC, add2(glp, glq));
-    cC = add2(cC, sub2(glp, glq));
-    if (fric) {
-        const float2 gadt = mul2(v2(-1.f), add2(gdp, gdq));
-        fric_adj1(gadt.x, C.w.x, C.t.x, C.e.x, C.d.x, s2.x, kf.x, clA, wC.x, tC.x, eC.x);
-        fric_adj1(gadt.y, C.w.y, C.t.y, C.e.y, C.d.y, s2.y, kf.y, clB, wC.y, tC.y, eC.y);
+    // the right interfaces: the adjoints of their two nodes together, then the transpose
+    const float2 A = mul2(make_float2(__fadd_rn(gRa.x, gLa.y), __fadd_rn(gRa.y, dn(gLa.x))), hr);
+    const float2 B = mul2(make_float2(__fadd_rn(gRb.x, gLb.y), __fadd_rn(gRb.y, dn(gLb.x))), hr);
+    const float2 T = mul2(make_float2(__fadd_rn(gRt.x, gLt.y), __fadd_rn(gRt.y, dn(gLt.x))), hr);
+    const float2 gdw = fma2(A, sw, mul2(B, sc));
+    const float2 gsw = fma2(A, dw, fma2(B, dc, mul2(T, dt)));
+    const float2 gnum = mul2(mul2(B, sw), rs);
+    float2 gsc = sub2(mul2(B, dw), mul2(gnum, dc));
+    float2 gdt = mul2(T, sw), gde = mul2(v2(2.f * GRAV), add2(A, gnum));
+    float2 rw = add2(gsw, gdw), lw = sub2(gsw, gdw);   // to w of the right and of the left node
+    if (edge) {
+        if (!inA) gsc.x = gdt.x = gde.x = rw.x = lw.x = 0.f;
+        if (!inB) gsc.y = gdt.y = gde.y = rw.y = lw.y = 0.f;
     }
-    if (SRC) {
-        const float2 gs = mul2(sub2(gdp, gdq), sdt);
-        cC = fma2(gs, C.w, cC);
-        wC = fma2(gs, C.c, wC);
-    }
-    float2 cL, cR;
-    {   // left interface: b = L, a = C
-        const float2 A = mul2(gQpL, il), B = mul2(gQqL, il), T = mul2(gQtL, il);
-        const float2 hp = fma2(v2(0.5f), fl.dw, fl.dcs), hq = fma2(v2(0.5f), fl.dw, mul2(v2(-1.f), fl.dcs));
-        const float2 sp = add2(fl.sw, fl.S), sq = sub2(fl.sw, fl.S);
-        const float2 hsp = mul2(v2(0.5f), sp), hsq = mul2(v2(0.5f), sq);
-        const float2 tdt = mul2(mul2(v2(0.5f), T), fl.dtt), tsw = mul2(mul2(v2(0.5f), T), fl.sw);
-        wC = add2(wC, fma2(A, add2(hp, hsp), fma2(B, add2(hq, hsq), tdt)));
-        bL[1] = fma2(A, sub2(hp, hsp), fma2(B, sub2(hq, hsq), tdt));
-        cC = add2(cC, sub2(mul2(A, add2(hp, sp)), mul2(B, add2(hq, sq))));
-        cL = sub2(mul2(A, sub2(hp, sp)), mul2(B, sub2(hq, sq)));
-        tC = add2(tC, tsw);
-        bL[2] = mul2(v2(-1.f), tsw);
-    }
-    {   // right interface: b = C, a = R
-        const float2 A = mul2(gQpR, ir), B = mul2(gQqR, ir), T = mul2(gQtR, ir);
-        const float2 hp = fma2(v2(0.5f), fr.dw, fr.dcs), hq = fma2(v2(0.5f), fr.dw, mul2(v2(-1.f), fr.dcs));
-        const float2 sp = add2(fr.sw, fr.S), sq = sub2(fr.sw, fr.S);
-        const float2 hsp = mul2(v2(0.5f), sp), hsq = mul2(v2(0.5f), sq);
-        const float2 tdt = mul2(mul2(v2(0.5f), T), fr.dtt), tsw = mul2(mul2(v2(0.5f), T), fr.sw);
-        bR[1] = fma2(A, add2(hp, hsp), fma2(B, add2(hq, hsq), tdt));
-        wC = add2(wC, fma2(A, sub2(hp, hsp), fma2(B, sub2(hq, hsq), tdt)));
-        cR = sub2(mul2(A, add2(hp, sp)), mul2(B, add2(hq, sq)));
-        cC = add2(cC, sub2(mul2(A, sub2(hp, sp)), mul2(B, sub2(hq, sq))));
-        bR[2] = tsw;
-        tC = sub2(tC, tsw);
-    }
-    const float2 hg = v2(0.5f * GRAV);
-    bC[0] = fma2(mul2(cC, hg), rcp2(C.c), eC);
-    bC[1] = wC;
-    bC[2] = tC;
-    bL[0] = mul2(mul2(cL, hg), rcp2(L.c));
-    bR[0] = mul2(mul2(cR, hg), rcp2(R.c));
+    auto sh = [&](float2 x) { return make_float2(up(x.y), x.x); };             // from the left interface
+    cC = add2(add2(cC, gsc), sh(gsc));
+    oe = fma2(mul2(cC, v2(0.5f * GRAV)), rc, add2(sub2(eC, gde), sh(gde)));
+    ow = add2(add2(wC, lw), sh(rw));
+    ot = add2(sub2(tC, gdt), sh(gdt));
 }
 
 // neighbours across the window: node 0 of a lane is window node 2*lane, node 1 is 2*lane+1
@@ -384,13 +355,14 @@ __device__ __forceinline__ void nbr(const int (&x)[2], int (&l)[2], int (&r)[2])
 // Adjoint of one sweep of a 64-node line window. In: the sweep's input (e, w, t, d) and the
 // adjoint (ge, gw, gt) of its output. Out: the adjoint of its input, exact at window
 // nodes 6..57.
-// ends: this lane's nodes at open outer edges, bits 1 node 0 left, 2 node 0 right, 4 node 1
+// pA: the lane's first node on a line of npos. ends: this lane's nodes at open outer edges, bits 1 node 0 left, 2 node 0 right, 4 node 1
 // left, 8 node 1 right (their outside neighbour is the open ghost instead of a mirror).
 template <bool SRC, bool S1>
 __device__ __forceinline__ void line_adjoint(const float (&e)[2], const float (&w)[2], const float (&t)[2],
                                              const float (&d)[2], const float (&ge)[2], const float (&gw)[2],
                                              const float (&gt)[2], const AMet (&m)[2], const SweepConst& K,
-                                             float (&oe)[2], float (&ow)[2], float (&ot)[2], unsigned ends = 0u) {
+                                             float (&oe)[2], float (&ow)[2], float (&ot)[2], unsigned ends, int pA,
+                                             int npos) {
     // (a) wet marks at the start of the sweep
     int o[2], fl[2];
 #pragma unroll
@@ -398,28 +370,21 @@ __device__ __forceinline__ void line_adjoint(const float (&e)[2], const float (&
         fl[i] = d[i] >= K.dwall;
         o[i] = fl[i] && (e[i] + d[i] >= K.hmin);
     }
-    if (!S1 && __all_sync(FULL, o[0] && o[1])) {
-        // every node of the window wet: no (b), no walls, no (e); only the stencil of (d)
-        float c[2];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) c[i] = wave_speed(e[i] + d[i]);
-        float eL[2], eR[2], wL[2], wR[2], tL[2], tR[2], dL[2], dR[2], cL[2], cR[2];
-        nbr(e, eL, eR); nbr(w, wL, wR); nbr(t, tL, tR); nbr(d, dL, dR); nbr(c, cL, cR);
+    // every node of the window that lies on the line wet (and no open edge): no (b), no (e), walls
+    // only at the line's ends
+    const bool in0 = pA >= 0 && pA < npos, in1 = pA + 1 >= 0 && pA + 1 < npos;
+    if (!S1 && __all_sync(FULL, (o[0] || !in0) && (o[1] || !in1) && !ends)) {
         auto f2 = [](const float (&x)[2]) { return make_float2(x[0], x[1]); };
-        const N2 Ln{f2(eL), f2(wL), f2(tL), f2(dL), f2(cL)}, Cn{f2(e), f2(w), f2(t), f2(d), f2(c)};
-        const N2 Rn{f2(eR), f2(wR), f2(tR), f2(dR), f2(cR)};
-        float2 bL[3], bC[3], bR[3];
-        a_dstage_adj2<SRC>(Ln, Cn, Rn, make_float2(m[0].il, m[1].il), make_float2(m[0].ir, m[1].ir),
-                           make_float2(m[0].k2, m[1].k2), make_float2(m[0].sdt, m[1].sdt), K, f2(ge), f2(gw),
-                           f2(gt), bL, bC, bR);
-        // node A gathers from B's left part and lane-1's B's right part; B from A's right
-        // part and lane+1's A's left part
-        float* out[3] = {oe, ow, ot};
-#pragma unroll
-        for (int f = 0; f < 3; ++f) {
-            out[f][0] = bC[f].x + bL[f].y + __shfl_up_sync(FULL, bR[f].y, 1);
-            out[f][1] = bC[f].y + bR[f].x + __shfl_down_sync(FULL, bL[f].x, 1);
-        }
+        const bool edge = !__all_sync(FULL, in0 && in1) || npos <= XWIN;
+        float2 e2, w2, t2;
+        line_adjoint_open<SRC>(f2(e), f2(w), f2(t), f2(d), f2(ge), f2(gw), f2(gt), make_float2(m[0].hl, m[1].hl),
+                               make_float2(m[0].hr, m[1].hr), make_float2(m[0].k2, m[1].k2),
+                               make_float2(m[0].nsdt, m[1].nsdt), K, edge, pA == 0,
+                               pA == npos - 1 ? 1 : pA + 1 == npos - 1 ? 2 : 0, in0 && in1, in1 && pA + 2 < npos,
+                               e2, w2, t2);
+        oe[0] = e2.x; oe[1] = e2.y;
+        ow[0] = w2.x; ow[1] = w2.y;
+        ot[0] = t2.x; ot[1] = t2.y;
         return;
     }
     // (b) flooding from the wetter neighbour (left on a tie), start-of-sweep values
@@ -596,10 +561,10 @@ __global__ void __launch_bounds__(AWARPS * 32, SPH ? 2 : CLIFFS_ADJ_LINE_BLOCKS)
         const int p = pA + i;
         mb[i] = AMet{0.f, 0.f, 0.f, 0.f};
         if (DIR == 0) {
-            if (p >= 0 && p < A.npos) mb[i] = AMet{2.f * A.xa[p], 2.f * A.xb[p], A.xk[p], 0.f};
+            if (p >= 0 && p < A.npos) mb[i] = AMet{A.xa[p], A.xb[p], A.xk[p], 0.f};
         } else {
             const float4 q = A.ymet[min(max(p, -MET_PAD), A.npos - 1 + MET_PAD)];
-            mb[i] = AMet{2.f * q.x, 2.f * q.y, q.z, -q.w};
+            mb[i] = AMet{q.x, q.y, q.z, q.w};
         }
     }
     static_assert(ALINES == AWARPS, "one line per warp");
@@ -632,7 +597,7 @@ __global__ void __launch_bounds__(AWARPS * 32, SPH ? 2 : CLIFFS_ADJ_LINE_BLOCKS)
         if (DIR == 0 && SPH) {
             const float f = A.xrow[line];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) { m[i].il *= f; m[i].ir *= f; m[i].k2 *= f; }
+            for (int i = 0; i < 2; ++i) { m[i].hl *= f; m[i].hr *= f; m[i].k2 *= f; }
         }
         float oe[2], ow[2], ot[2];
         unsigned ends = 0u;
@@ -640,7 +605,7 @@ __global__ void __launch_bounds__(AWARPS * 32, SPH ? 2 : CLIFFS_ADJ_LINE_BLOCKS)
             if (A.open_lo) ends |= (pA == 0 ? 1u : 0u) | (pA + 1 == 0 ? 4u : 0u);
             if (A.open_hi) ends |= (pA == A.npos - 1 ? 2u : 0u) | (pA + 1 == A.npos - 1 ? 8u : 0u);
         }
-        line_adjoint<DIR == 1 && SPH, S1>(e, w, t, d, ge, gw, gt, m, K, oe, ow, ot, ends);
+        line_adjoint<DIR == 1 && SPH, S1>(e, w, t, d, ge, gw, gt, m, K, oe, ow, ot, ends, pA, A.npos);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const int q = 2 * lane + i - AHALO;

@@ -361,7 +361,7 @@ int cliffs_kernel_time(cliffs_grid* g, int enable, double* ms, int64_t* launches
  * forbids allocations behind its back (a hidden allocation can fail, or fragment the pool),
  * and callers that cannot afford cudaFree's device-wide synchronisation, which stalls every
  * stream on the device. It allocates nothing: its scratch (a second FP64 Jacobi buffer and
- * a flag) is one static device array of CLIFFS_NOALLOC_MAX_CELLS doubles (8 MiB) that every
+ * the passes' flags) is one static device array of CLIFFS_NOALLOC_MAX_CELLS doubles (8 MiB) that every
  * GPU loading the library holds until the process exits.
  *   depth   [ny][nx] FP64 input depth, positive down (host or device memory)
  *   out     [ny][nx] FP64 filtered depth, DEVICE (or managed) memory owned by the caller;
@@ -377,8 +377,9 @@ int cliffs_kernel_time(cliffs_grid* g, int enable, double* ms, int64_t* launches
  * (cudaGetSymbolAddress) with that device current and keeps it; make that first call before
  * any stream capture. The kept address does not survive cudaDeviceReset. Every call on a
  * device shares the one array and leaves its last contents there (the flag is cleared
- * before each pass): calls that overlap on the GPU (other streams or threads) race and give
- * wrong results. The call synchronises the stream once per pass to read the flag. */
+ * before each call): calls that overlap on the GPU (other streams or threads) race and give
+ * wrong results. The call synchronises the stream once per group of passes (8, 16, 32, 44) to read
+ * the flags. */
 #define CLIFFS_NOALLOC_MAX_CELLS (1 << 20)
 int cliffs_depth_filter_noalloc(const double* depth, double* out, int32_t nx, int32_t ny,
                                 double alpha, double min_depth, void* stream, int32_t* passes);

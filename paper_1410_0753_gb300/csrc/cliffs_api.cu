@@ -21,6 +21,7 @@
 #include "cliffs.h"
 #include "internal.h"
 #include "adjoint.h"
+#include "filter.cuh"
 #include "sweep.cuh"
 
 using namespace cliffs;
@@ -66,19 +67,6 @@ const int ADJ_GROUP_WAVES = CLIFFS_ADJ_GROUP_WAVES;
 const bool ADJ_PDL = CLIFFS_ADJ_PDL != 0;     // programmatic launches between the adjoint's kernels
 
 // ----------------------------------------------------------------------------- kernels
-
-// depth-jump filter, section "Numerical stability": eqs. (dstab), (newdw), (newdc)
-__global__ void k_filter_minraise(double* d, long long n, double min_depth) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i < n) filter_minraise_node(d, i, min_depth);
-}
-
-// One Jacobi pass along rows (dir 0) or columns (dir 1).
-__global__ void k_filter_pass(const double* in, double* out, int nx, int ny, int dir, double a2,
-                              int* changed) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i < (long long)nx * ny) filter_pass_node(in, out, i, nx, ny, dir, a2, changed);
-}
 
 __global__ void k_depth_to_f32(const double* d64, float* d32, int nx, int ny, int pitch) {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -994,7 +982,7 @@ int cliffs_grid_create(const cliffs_config* cfg, cliffs_grid** out) {
     CKG(cudaMalloc(&g->ymp, sizeof(float4) * (ny + 2 * MET_PAD)));
     CKG(cudaMalloc(&g->err, sizeof(int) * 4));
     CKG(cudaMemsetAsync(g->err, 0, sizeof(int) * 4, g->stream));
-    CKG(cudaMalloc(&g->ured, sizeof(unsigned) * 4));
+    CKG(cudaMalloc(&g->ured, sizeof(unsigned) * FILTER_PASSES));
     CKG(cudaStreamSynchronize(g->stream));
 #undef CKG
     if (nx >= 3 && ny >= 3) {
@@ -1029,22 +1017,11 @@ int cliffs_set_bathy(cliffs_grid* g, const double* x, const double* y, const dou
     cudaStream_t s = g->stream;
     CK(cudaMemcpyAsync(g->d64, depth, sizeof(double) * N, cudaMemcpyDefault, s));
     if (apply_filter) {
-        k_filter_minraise<<<nblk(N), 256, 0, s>>>(g->d64, N, min_depth);
+        k_filter_raise<<<nblk(N), 256, 0, s>>>(g->d64, g->d64, N, min_depth);
         CK(cudaGetLastError());
-        int* changed = reinterpret_cast<int*>(g->ured);
-        const double a2 = alpha * alpha;
-        bool conv = false;
-        for (int pass = 1; pass <= 100; ++pass) {
-            CK(cudaMemsetAsync(changed, 0, sizeof(int), s));
-            k_filter_pass<<<nblk(N), 256, 0, s>>>(g->d64, g->d64b, nx, ny, 0, a2, changed);
-            k_filter_pass<<<nblk(N), 256, 0, s>>>(g->d64b, g->d64, nx, ny, 1, a2, changed);
-            CK(cudaGetLastError());
-            int h = 0;
-            CK(cudaMemcpyAsync(&h, changed, sizeof(int), cudaMemcpyDeviceToHost, s));
-            CK(cudaStreamSynchronize(s));
-            if (!h) { conv = true; break; }
-        }
-        if (!conv) fprintf(stderr, "cliffs: depth filter stopped after 100 passes\n");
+        int passes = 0;
+        CK(run_filter(g->d64, g->d64b, nx, ny, alpha, reinterpret_cast<int*>(g->ured), s, &passes));
+        if (passes < 0) fprintf(stderr, "cliffs: depth filter stopped after 100 passes\n");
     }
     // metric tables (section "Running Options", "Units": metres, or degrees on a sphere)
     std::vector<float> xa(nx, 0.f), xb(nx, 0.f), xk(nx, 0.f), xrow(ny, 1.f);

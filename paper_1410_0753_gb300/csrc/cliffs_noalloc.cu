@@ -2,38 +2,28 @@
 //
 // Same filter as cliffs_set_bathy's (wet nodes raised to min_depth, then row and column
 // Jacobi passes of eqs. (dstab), (newdw), (newdc) until a pass changes nothing, at most
-// 100), but its scratch (the second Jacobi buffer and the "changed" flag) is a fixed static
+// 100), but its scratch (the second Jacobi buffer and the "changed" flags) is a fixed static
 // device array instead of memory from cudaMalloc, and it writes into memory the caller owns.
 // Nothing here calls cudaMalloc, cudaFree or any allocating library routine.
 #include <cstdio>
 #include <mutex>
 
 #include "cliffs.h"
+#include "filter.cuh"
 #include "internal.h"
 
 namespace {
 
 // The scratch every device that loads the library keeps until exit: the first 256 bytes
-// hold the "changed" flag, the rest one FP64 Jacobi buffer of up to
+// hold the passes' "changed" flags, the rest one FP64 Jacobi buffer of up to
 // CLIFFS_NOALLOC_MAX_CELLS nodes.
-constexpr int FLAG_SLOTS = 32;   // 256 bytes
+constexpr int FLAG_SLOTS = 64;   // 512 bytes
+static_assert(FLAG_SLOTS * 2 >= cliffs::FILTER_PASSES, "one int per pass");
 static __device__ __align__(256) double g_scratch[FLAG_SLOTS + CLIFFS_NOALLOC_MAX_CELLS];
 
 std::mutex g_mu;
 constexpr int MAX_DEVICES = 64;
 double* g_dev_ptr[MAX_DEVICES] = {nullptr};
-
-// The same per-node code as cliffs_set_bathy's filter kernels (internal.h).
-__global__ void k_na_minraise(double* d, long long n, double min_depth) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i < n) cliffs::filter_minraise_node(d, i, min_depth);
-}
-
-__global__ void k_na_pass(const double* in, double* out, int nx, int ny, int dir, double a2,
-                          int* changed) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i < (long long)nx * ny) cliffs::filter_pass_node(in, out, i, nx, ny, dir, a2, changed);
-}
 
 // Memory type of a pointer as the runtime sees it (cudaMemoryTypeUnregistered for plain
 // host memory it does not know).
@@ -111,27 +101,17 @@ int cliffs_depth_filter_noalloc(const double* depth, double* out, int32_t nx, in
     double* tmp = base + FLAG_SLOTS;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const unsigned blocks = (unsigned)((N + 255) / 256);
-    if (out != depth) {
+    const double* src = depth;
+    if (out != depth && ti != cudaMemoryTypeDevice && ti != cudaMemoryTypeManaged) {
         e = cudaMemcpyAsync(out, depth, sizeof(double) * N, cudaMemcpyDefault, s);
         if (e != cudaSuccess) return fail(CLIFFS_ERR_CUDA, "copy of the input depth", e);
+        src = out;
     }
-    k_na_minraise<<<blocks, 256, 0, s>>>(out, N, min_depth);
-    const double a2 = alpha * alpha;
-    int pass = 1;
-    for (; pass <= 100; ++pass) {
-        e = cudaMemsetAsync(changed, 0, sizeof(int), s);          // the flag starts at zero
-        if (e != cudaSuccess) return fail(CLIFFS_ERR_CUDA, "flag reset", e);
-        k_na_pass<<<blocks, 256, 0, s>>>(out, tmp, nx, ny, 0, a2, changed);
-        k_na_pass<<<blocks, 256, 0, s>>>(tmp, out, nx, ny, 1, a2, changed);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return fail(CLIFFS_ERR_CUDA, "filter pass launch", e);
-        int h = 0;
-        e = cudaMemcpyAsync(&h, changed, sizeof(int), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) return fail(CLIFFS_ERR_CUDA, "flag read", e);
-        if (!h) break;
-    }
-    if (passes) *passes = pass <= 100 ? pass : -1;
+    cliffs::k_filter_raise<<<blocks, 256, 0, s>>>(src, out, N, min_depth);
+    int made = 0;
+    e = cliffs::run_filter(out, tmp, nx, ny, alpha, changed, s, &made);
+    if (e != cudaSuccess) return fail(CLIFFS_ERR_CUDA, "filter passes", e);
+    if (passes) *passes = made;
     return CLIFFS_OK;
 }
 

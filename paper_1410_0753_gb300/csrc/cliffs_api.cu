@@ -336,6 +336,7 @@ struct cliffs_grid {
     std::vector<unsigned char> hard;         // [nstrips][ny]: dry nodes in the strip's window within 3 rows
     std::vector<double> strip_cost;          // per strip: the cost of its rows (item_cost)
     ItemSet march, tile;                     // work items of the fused kernel (1D: samples only) and of the tiles
+    ItemSet batch;                           // and of the persistent run by marching warps, made when first needed
     int tile_R = 0, tile_rows = 0;           // rows per tile in open water; the largest tile with its halo
     bool S_set = false;                      // S was set or tuned by the caller: steps march
     // timing
@@ -612,6 +613,26 @@ bool by_tiles(const cliffs_grid* g) {
     return g->kind == 0 && !g->S_set && (long long)g->tile.items.size() * g->B <= 2ll * num_sms();
 }
 
+// Rows per warp of the persistent run by marching warps: its items are handed out in rounds of
+// the resident warps, so the smallest sum of rounds * (rows + 3.7) counts, over batches that
+// shrink as scenarios end (all of them running, three quarters, half, a quarter). 48 scenarios
+// of 512^2, all running: 95.5 us per step at 28 rows, 109 at 24, 103 at 40, 131 at 20 (the choice
+// for one launch per step).
+int choose_batch(cliffs_grid* g) {
+    const long long resident = resident_warps(g);
+    double best = 1e300;
+    int bestS = 32;
+    for (int S = 4; S <= 128 && S <= std::max(4, g->ny); S += 2) {
+        const long long n1 = fused_warps(g, S) / g->B;
+        double cost = 0.0;
+        for (int q = 4; q >= (g->B >= 4 ? 1 : 4); --q)
+            cost += (double)((n1 * ((g->B * q + 3) / 4) + resident - 1) / resident) * (S + 3.7);
+        if (cost < best) { best = cost; bestS = S; }
+    }
+    cut_items(g, bestS, g->batch.items);
+    return upload_items(g, g->batch);
+}
+
 int choose_geometry(cliffs_grid* g) {
     if (g->ny == 1) {
         g->kind = 1;
@@ -639,6 +660,7 @@ int choose_geometry(cliffs_grid* g) {
         const int rc = set_rows_per_warp(g, bestS);
         if (rc) return rc;
         g->S_set = false;
+        g->batch.items.clear();
         return choose_tile(g);
     }
     return build_samples(g, g->march);
@@ -726,12 +748,11 @@ int make_maps(cliffs_grid* g) {
     return CLIFFS_OK;
 }
 
-// the step by tiles in place of marching warps
-void use_tiles(const cliffs_grid* g, StepArgs& a) {
-    a.items = g->tile.dev;
-    a.nitems = (int)g->tile.items.size();
-    a.samp_ptr = g->tile.samp_ptr;
-    a.samp = g->tile.samp;
+void use_items(const ItemSet& set, StepArgs& a) {
+    a.items = set.dev;
+    a.nitems = (int)set.items.size();
+    a.samp_ptr = set.samp_ptr;
+    a.samp = set.samp;
 }
 
 void fill_step_args(cliffs_grid* g, StepArgs& a, int in, int out) {
@@ -871,7 +892,7 @@ void free_grid(cliffs_grid* g) {
     cudaFree(g->emax);
     cudaFree(g->xa); cudaFree(g->xb); cudaFree(g->xk); cudaFree(g->xrow); cudaFree(g->ymet); cudaFree(g->ymp);
     cudaFree(g->err); cudaFree(g->limit); cudaFree(g->items_d);
-    for (ItemSet* t : {&g->march, &g->tile}) { cudaFree(t->dev); cudaFree(t->samp_ptr); cudaFree(t->samp); }
+    for (ItemSet* t : {&g->march, &g->tile, &g->batch}) { cudaFree(t->dev); cudaFree(t->samp_ptr); cudaFree(t->samp); }
     cudaFree(g->grec); cudaFree(g->nrec);
     cudaFree(g->pt_slot); cudaFree(g->pt_w); cudaFree(g->tmp); cudaFree(g->ured);
     cudaFree(g->order_d); cudaFree(g->nact_d); cudaFree(g->ctl_d);
@@ -1451,7 +1472,7 @@ int cliffs_step_n(cliffs_grid* g, int64_t n) {
         }
         cudaError_t le;
         if (tiles) {
-            use_tiles(g, a);
+            use_items(g->tile, a);
             le = launch_step_tile(a, g->B, s);
         } else if (g->kind == 0) le = launch_step_fused(a, g->maps[in], g->B, s);
         else if (g->kind == 1) le = launch_xsweep(a, g->B, s);
@@ -1512,16 +1533,21 @@ int cliffs_run_persistent(cliffs_grid* g, int64_t n) {
     }
     // no more blocks than the batch has work (each one more makes the barrier slower)
     const bool tiles = by_tiles(g);
-    const long long work = (tiles ? (long long)g->tile.items.size() : ((long long)g->march.items.size() + fused_warps_per_block() - 1) /
-                                                                          fused_warps_per_block()) * g->B;
+    if (!tiles && !g->S_set && g->batch.items.empty()) {
+        rc = choose_batch(g);
+        if (rc) return rc;
+    }
+    const ItemSet& set = tiles ? g->tile : g->S_set ? g->march : g->batch;
+    const long long per = tiles ? 1 : fused_warps_per_block();
+    const long long work = ((long long)set.items.size() * g->B + per - 1) / per;
     const int blocks = (int)std::min<long long>(tiles ? g->pblocks_tile : g->pblocks, work);
     // launch arguments; all padding zeroed so that they compare byte for byte
     struct Key { StepArgs a; BatchArgs b; long long tiles; } k;
     std::memset(&k, 0, sizeof(k));
     fill_step_args(g, k.a, 0, 1);
     k.a.eta_out = nullptr;
-    if (tiles) use_tiles(g, k.a);
-    else fused_ring(last >= g->cfg.maxout, &k.a.nslots, &k.a.slot_floats);
+    use_items(set, k.a);
+    if (!tiles) fused_ring(last >= g->cfg.maxout, &k.a.nslots, &k.a.slot_floats);
     k.tiles = tiles;
     k.a.eta_in = k.a.u_in = k.a.v_in = nullptr;
     k.a.limit = nullptr;

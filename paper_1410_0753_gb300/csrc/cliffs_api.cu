@@ -107,21 +107,41 @@ __global__ void k_quake(double* d64, const float* zeta, float* eta, float* d32, 
     d32[(long long)r * pitch + c] = (float)nd;
 }
 
-// max-wave initialisation from the state of step 0 (wet nodes), batched over planes
-__global__ void k_max_init(const float* eta, const float* u, const float* v, const float* d,
-                           float* emax, float* smax, int nx, int ny, int pitch, long long plane,
-                           int b0, int nb, float hmin, float dwall) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= (long long)nb * plane) return;
-    const long long o = (long long)b0 * plane + i;
-    const long long p = i % plane;
-    const int c = (int)(p % pitch);
-    const float dd = d[p];
-    const float e = eta[o];
-    const bool wet = c < nx && (dd >= dwall) && (e + dd >= hmin);
-    emax[o] = wet ? e : -3.402823466e38f;
-    smax[o] = wet ? sqrtf(u[o] * u[o] + v[o] * v[o]) : 0.f;
-    (void)ny;
+// The initial state of scenarios [b0, b0 + nb) and the max-wave fields that start from it (wet
+// nodes), in one pass: the dense [nb][ny][nx] eta (and u, v; null: at rest) into the pitched
+// planes. in_place: the planes hold the state already. 8192^2 from device memory, at rest:
+// 777 us as two-dimensional copies, clears and a pass of its own for the maxima, of which the
+// bytes moved once take 280.
+__global__ void __launch_bounds__(256) k_init_state(const float* __restrict__ eta, const float* __restrict__ u,
+                                                    const float* __restrict__ v, int in_place, float* st, long long fs,
+                                                    const float* __restrict__ d, float* emax, int nx, int ny, int pitch,
+                                                    long long plane, int b0, float hmin, float dwall) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= pitch) return;
+    for (int row = blockIdx.y; row < ny; row += gridDim.y) {
+        const int b = blockIdx.z;
+        const long long o = (b0 + b) * plane + (long long)row * pitch + c;
+        float e = 0.f, uu = 0.f, vv = 0.f;
+        if (in_place) {
+            e = st[o];
+            uu = st[fs + o];
+            vv = st[2 * fs + o];
+        } else {
+            if (c < nx) {
+                const long long i = ((long long)b * ny + row) * nx + c;
+                e = eta[i];
+                if (u) uu = u[i];
+                if (v) vv = v[i];
+            }
+            st[o] = e;
+            st[fs + o] = uu;
+            st[2 * fs + o] = vv;
+        }
+        const float dd = d[(long long)row * pitch + c];
+        const bool wet = c < nx && (dd >= dwall) && (e + dd >= hmin);
+        emax[o] = wet ? e : -3.402823466e38f;
+        emax[fs + o] = wet ? sqrtf(uu * uu + vv * vv) : 0.f;
+    }
 }
 
 // Diagnostics of one state plane (a monitor, not a step of the method): over wet nodes (the
@@ -407,6 +427,14 @@ struct cliffs_grid {
 };
 
 namespace {
+
+// whether p is memory of the current device (kernels may read it), rather than host or managed
+bool on_device(const void* p) {
+    cudaPointerAttributes at;
+    int dev = -1;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return false; }
+    return at.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess && at.device == dev;
+}
 
 int ensure_tmp(cliffs_grid* g, size_t bytes) {
     if (bytes <= g->tmp_bytes) return CLIFFS_OK;
@@ -1236,19 +1264,26 @@ int cliffs_set_initial(cliffs_grid* g, int scenario, const float* eta, const flo
         k_quake<<<nblk((long long)nx * ny), 256, 0, s>>>(g->d64, (const float*)g->tmp, g->eta[0], g->d32, nx, ny,
                                                         g->pitch, g->cfg.h_min, dwall);
         CK(cudaGetLastError());
-    } else {
-        CK(cudaMemcpy2DAsync(g->eta[0] + off, pitchb, eta, rowb, rowb, rows, cudaMemcpyDefault, s));
     }
-    if (u) CK(cudaMemcpy2DAsync(g->u[0] + off, pitchb, u, rowb, rowb, rows, cudaMemcpyDefault, s));
-    else CK(cudaMemsetAsync(g->u[0] + off, 0, sizeof(float) * nb * g->plane, s));
-    if (v) CK(cudaMemcpy2DAsync(g->v[0] + off, pitchb, v, rowb, rowb, rows, cudaMemcpyDefault, s));
-    else CK(cudaMemsetAsync(g->v[0] + off, 0, sizeof(float) * nb * g->plane, s));
+    // fields in device memory are read where they are; anything else is copied into the planes
+    const bool direct = !quake && on_device(eta) && (!u || on_device(u)) && (!v || on_device(v));
+    if (!direct) {
+        if (!quake) CK(cudaMemcpy2DAsync(g->eta[0] + off, pitchb, eta, rowb, rowb, rows, cudaMemcpyDefault, s));
+        if (u) CK(cudaMemcpy2DAsync(g->u[0] + off, pitchb, u, rowb, rowb, rows, cudaMemcpyDefault, s));
+        else CK(cudaMemsetAsync(g->u[0] + off, 0, sizeof(float) * nb * g->plane, s));
+        if (v) CK(cudaMemcpy2DAsync(g->v[0] + off, pitchb, v, rowb, rowb, rows, cudaMemcpyDefault, s));
+        else CK(cudaMemsetAsync(g->v[0] + off, 0, sizeof(float) * nb * g->plane, s));
+    }
     g->step = 0;
     const float dwall = g->cfg.itopo ? -3.402823466e38f : (float)g->cfg.dwall;
-    k_max_init<<<nblk((long long)nb * g->plane), 256, 0, s>>>(g->eta[0], g->u[0], g->v[0], g->d32, g->emax, g->smax,
-                                                             nx, ny, g->pitch, g->plane, b0, nb,
-                                                             (float)g->cfg.h_min, dwall);
-    CK(cudaGetLastError());
+    for (int z = 0; z < nb; z += 32768) {
+        const int m = std::min(nb - z, 32768);
+        const long long i = (long long)z * ny * nx;
+        k_init_state<<<dim3((g->pitch + 255) / 256, std::min(ny, 32768), m), 256, 0, s>>>(
+            direct ? eta + i : nullptr, direct && u ? u + i : nullptr, direct && v ? v + i : nullptr, !direct, g->st[0],
+            (long long)g->B * g->plane, g->d32, g->emax, nx, ny, g->pitch, g->plane, b0 + z, (float)g->cfg.h_min, dwall);
+        CK(cudaGetLastError());
+    }
     int rc = grow_records(g, 1, 1);
     if (rc) return rc;
     if (!g->samples.empty()) {

@@ -813,6 +813,7 @@ void fill_step_args(cliffs_grid* g, StepArgs& a, int in, int out) {
     a.sph = g->cfg.coords != 1;
     a.wait_cycles = 2000000000LL;            // about a second at the GB300's clocks
     a.tx_pad = 0;
+    a.bnd = 0;
     a.walls = g->cfg.itopo == 0;
     fused_ring(false, &a.nslots, &a.slot_floats);
     a.yfirst = 0;
@@ -1459,7 +1460,7 @@ int cliffs_step_n(cliffs_grid* g, int64_t n) {
     int rc = grow_records(g, last / g->cfg.gout + 1, last / g->cfg.bndout + 1);
     if (rc) return rc;
     cudaStream_t s = g->stream;
-    StepArgs a;
+    StepArgs a{};
     const bool tiles = by_tiles(g) && g->inject_cycles <= 0;
     // A run recorded with every state kept (checkpoint j is the state after j steps, laid out as
     // a state buffer): the tile kernel steps from checkpoint to checkpoint, and the last one is
@@ -1499,10 +1500,17 @@ int cliffs_step_n(cliffs_grid* g, int64_t n) {
         if (g->bnd_any) {
             const double t = bnd_time(g, g->step);
             if (bnd_stops(g, t, t_end)) break;
-            rc = impose_boundary(g, g->eta[in], g->u[in], g->v[in], t);
-            if (rc) return rc;
+            if (!tiles) {
+                rc = impose_boundary(g, g->eta[in], g->u[in], g->v[in], t);
+                if (rc) return rc;
+            }
         }
         fill_step_args(g, a, in, out);
+        if (g->bnd_any && tiles) {                           // the tile kernel takes the input as it reads
+            a.bnd = 1;
+            a.bnd_row = bnd_row(g, bnd_time(g, g->step));
+            for (int e = 0; e < 4; ++e) a.bnd_vals[e] = g->bnd_t[e].empty() ? nullptr : g->bnd_v[e];
+        }
         a.step = st;
         a.yfirst = g->cfg.alternate && ((st - 1) & 1);       // odd steps sweep y first
         if (st % g->cfg.maxout == 0) a.emax = g->emax;
@@ -1645,6 +1653,7 @@ int cliffs_run_persistent(cliffs_grid* g, int64_t n) {
         b.bnd = 1;
         b.bnd_rows = g->bnd_rows;
         for (int e = 0; e < 4; ++e) {
+            if (tiles) k.a.bnd_vals[e] = g->bnd_t[e].empty() ? nullptr : g->bnd_v[e];
             b.bv[e] = g->bnd_t[e].empty() ? nullptr : g->bnd_v[e];
             b.bnp[e] = e < 2 ? g->ny : g->nx;
         }
@@ -1931,7 +1940,7 @@ static int adjoint_core(cliffs_grid* g, int scenario, int64_t n, int32_t checkpo
     float* DT = g->adj_t + 6 * TPL;                         // depth transposed
     float* LB = g->adj_lb;                                  // adjoint (eta, u, v) row-major
     auto slot = [&](int j) { return g->adj_slots + 3 * FS * j; };
-    StepArgs a;
+    StepArgs a{};
     fill_step_args(g, a, 0, 1);
     a.limit = nullptr;
     a.step = 1;
@@ -2214,7 +2223,7 @@ int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32
     CK(cudaMalloc(&scratch, 3 * pb + flush_bytes));
     unsigned char* flush = reinterpret_cast<unsigned char*>(scratch + 3 * (pb / sizeof(float)));
     const int cur = (int)(g->step & 1);
-    StepArgs a;
+    StepArgs a{};
     fill_step_args(g, a, cur, 1 - cur);
     a.eta_out = scratch;
     a.step = g->step + 1;

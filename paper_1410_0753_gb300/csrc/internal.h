@@ -21,6 +21,12 @@ struct SweepConst {
     float2 lgf;       // log2(dt g n^2 g^(4/3)) (friction, fric_k2)
 };
 
+// Interpolation of one step's boundary input per edge: record k and weight w toward k + 1.
+struct BndRow {
+    long long k[4];
+    double w[4];
+};
+
 // Arguments of one sweep-kernel launch (all device pointers). Fields 2D are pitched:
 // element (b, r, c) lives at b * plane + r * pitch + c.
 struct StepArgs {
@@ -57,6 +63,10 @@ struct StepArgs {
     int sph;                         // geographic grid: x metric scaled per row
     int yfirst;                      // this step sweeps y, then x (alternating order)
     int open_edges;                  // open outer edges: bits W 1, E 2, S 4, N 8
+    // boundary input, taken by the tile kernels as they read the state (bnd: this launch's step)
+    int bnd;
+    BndRow bnd_row;
+    const double* bnd_vals[4];       // records [nt][3][np] per edge, or null
     long long wait_cycles;           // limit of every mbarrier wait (clock cycles)
     unsigned tx_pad;                 // extra bytes each ring slot expects (fault injection; 0)
 };
@@ -83,12 +93,6 @@ struct StepMaps2 {
 // The batched persistent run (k_batch, k_batch_tile). ctl lives in device memory so that one captured
 // graph serves every call: ctl[0] = steps done before the launch, ctl[1] = steps done after
 // it, ctl[2] = grid barrier (arrival count in the low 32 bits, generation in the high 32).
-// Interpolation of one step's boundary input per edge: record k and weight w toward k + 1.
-struct BndRow {
-    long long k[4];
-    double w[4];
-};
-
 struct BatchArgs {
     long long* ctl;
     const int* order;                // scenarios by decreasing step limit
@@ -111,27 +115,37 @@ struct BatchArgs {
     int bnp[4];                      // nodes per edge
 };
 
-// Edge node q of edge e (0 W, 1 E, 2 S, 3 N) takes its input (u, v, eta) from record k with
-// weight w toward k + 1 (the interpolation in FP64, non-fused, then rounded to FP32). S and
-// N own the corners when they carry input. Shared by the per-step kernel and the persistent
-// one, so both give the same bits.
+// The input (u, v, eta) of edge node q of edge e (0 W, 1 E, 2 S, 3 N; n nodes) from record k with
+// weight w toward k + 1 (the interpolation in FP64, non-fused, then rounded to FP32). Shared by
+// the per-step kernel and those that take it as they read, so all give the same bits.
+__device__ __forceinline__ float bnd_value(const double* vals, int n, int f, int q, long long k, double w) {
+    const double* r0 = vals + k * 3 * n;
+    const double a = r0[f * n + q];
+    return (float)((w > 0.0) ? __dadd_rn(__dmul_rn(__dsub_rn(1.0, w), a), __dmul_rn(w, r0[(3 + f) * n + q])) : a);
+}
+// Edge node q of edge e takes its input. S and N own the corners when they carry input.
 __device__ __forceinline__ void bnd_apply(float* eta, float* u, float* v, int pitch, int nx, int ny, int e, int q,
                                           const double* const* vals, const int* np, long long k, double w) {
     if (!vals[e] || q >= np[e]) return;
     if (e < 2 && ((q == 0 && vals[2]) || (q == ny - 1 && vals[3])) && nx > 1 && ny > 1) return;
     const int ix = (e == 0) ? 0 : (e == 1) ? nx - 1 : q;
     const int iy = (e == 2) ? 0 : (e == 3) ? ny - 1 : q;
-    const int n = np[e];
-    const double* r0 = vals[e] + k * 3 * n;
-    double val[3];
-    for (int f = 0; f < 3; ++f) {
-        const double a = r0[f * n + q];
-        val[f] = (w > 0.0) ? __dadd_rn(__dmul_rn(__dsub_rn(1.0, w), a), __dmul_rn(w, r0[(3 + f) * n + q])) : a;
-    }
     const size_t o = (size_t)iy * pitch + ix;
-    u[o] = (float)val[0];
-    v[o] = (float)val[1];
-    eta[o] = (float)val[2];
+    u[o] = bnd_value(vals[e], np[e], 0, q, k, w);
+    v[o] = bnd_value(vals[e], np[e], 1, q, k, w);
+    eta[o] = bnd_value(vals[e], np[e], 2, q, k, w);
+}
+// Node (iy, ix) as a step reads it under boundary input: its edge's input, else (e, u, v) as
+// they are.
+__device__ __forceinline__ void bnd_read(float& e, float& u, float& v, int nx, int ny, int ix, int iy,
+                                         const double* const* vals, const BndRow& R) {
+    const int g = (iy == 0 && vals[2]) ? 2 : (iy == ny - 1 && vals[3]) ? 3 : (ix == nx - 1 && vals[1]) ? 1 :
+                  (ix == 0 && vals[0]) ? 0 : -1;
+    if (g < 0) return;
+    const int n = g < 2 ? ny : nx, q = g < 2 ? iy : ix;
+    u = bnd_value(vals[g], n, 0, q, R.k[g], R.w[g]);
+    v = bnd_value(vals[g], n, 1, q, R.k[g], R.w[g]);
+    e = bnd_value(vals[g], n, 2, q, R.k[g], R.w[g]);
 }
 
 // launchers (cliffs_step.cu, cliffs_tile.cu)

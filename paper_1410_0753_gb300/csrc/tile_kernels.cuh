@@ -34,6 +34,7 @@ struct Tile {
     XMet2 m0;
     YMarch2 ym;
     StepOut O;
+    const BndRow* bnd;         // this step's boundary input, or null
     const float* in;           // eta of the input state (this lane's pair of row 0); u, v at fs_in
     int bad;
     float2 chk_x, chk_out;     // as in FusedWarp
@@ -106,6 +107,11 @@ struct Tile {
             U = ld_cg(in + a.fs_in + o);
             V = ld_cg(in + 2 * a.fs_in + o);
             D = __ldg(reinterpret_cast<const float2*>(a.d + o + c0 + 2 * lane));
+            if (bnd && (wallx || k == 0 || k == a.ny - 1)) {
+                const int cA = c0 + 2 * lane;
+                bnd_read(E.x, U.x, V.x, a.nx, a.ny, cA, k, a.bnd_vals, *bnd);
+                if (colB) bnd_read(E.y, U.y, V.y, a.nx, a.ny, cA + 1, k, a.bnd_vals, *bnd);
+            }
             if (!colB) { E.y = U.y = V.y = 0.f; D.y = OUTSIDE_D; }
         }
     }
@@ -248,8 +254,9 @@ struct Tile {
     }
 
     // item idx of scenario b_ (whole block)
-    __device__ __forceinline__ void run_item(int idx, int b_, const StepOut& O_, const float* eta_in) {
+    __device__ __forceinline__ void run_item(int idx, int b_, const StepOut& O_, const float* eta_in, const BndRow* bnd_) {
         O = O_;
+        bnd = bnd_;
         b = b_;
         in = eta_in + ((long long)b * a.plane + c0 + 2 * lane);
         sweep_rows();
@@ -276,7 +283,7 @@ k_step_tile(const __grid_constant__ StepArgs a) {
     Tile<SPH, FRIC, YF, S1, OPEN> T(a);
     T.setup(smem_raw);
     T.take_item(blockIdx.x);
-    T.run_item(blockIdx.x, b, step_out(nullptr, a), a.eta_in);
+    T.run_item(blockIdx.x, b, step_out(nullptr, a), a.eta_in, a.bnd ? &a.bnd_row : nullptr);
     T.report();
 }
 
@@ -299,19 +306,7 @@ k_batch_tile(const __grid_constant__ StepArgs a, const __grid_constant__ BatchAr
     for (long long st = step0 + 1; st <= step_end; ++st) {
         const bool yf = ALT && (((st - 1) & 1) != 0);
         const bool odd = (st & 1) != 0;          // odd steps read buffer 0 and write buffer 1
-        if (B.bnd) {
-            // boundary input: the edge nodes of this step's input take the input at its model
-            // time, then every block waits so that no load reads an edge before it is set
-            const BndRow& R = B.bnd_rows[st - step0 - 1];
-            float* ei = odd ? B.eta[0] : B.eta[1];
-            const int per = 2 * a.ny + 2 * a.nx;
-            for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < per; idx += gridDim.x * blockDim.x) {
-                const int e = idx < a.ny ? 0 : idx < 2 * a.ny ? 1 : idx < 2 * a.ny + a.nx ? 2 : 3;
-                const int q = e == 0 ? idx : e == 1 ? idx - a.ny : e == 2 ? idx - 2 * a.ny : idx - 2 * a.ny - a.nx;
-                bnd_apply(ei, ei + a.fs_out, ei + 2 * a.fs_out, a.pitch, a.nx, a.ny, e, q, B.bv, B.bnp, R.k[e], R.w[e]);
-            }
-            if (!grid_sync(reinterpret_cast<unsigned long long*>(B.ctl + 2), arrivals, a.wait_cycles, a.err)) break;
-        }
+        const BndRow* bnd = B.bnd ? &B.bnd_rows[st - step0 - 1] : nullptr;
         const bool mx = st % B.maxout == 0;
         const StepOut O{nullptr, odd ? B.eta[1] : B.eta[0], mx ? B.emax : nullptr,
                         (B.grec && st % B.gout == 0) ? B.grec + (st / B.gout) * B.grec_row : nullptr,
@@ -327,8 +322,8 @@ k_batch_tile(const __grid_constant__ StepArgs a, const __grid_constant__ BatchAr
                 taken = item;
             }
             if (t != blockIdx.x) __syncthreads();    // the tile before is done with shared memory
-            if (yf) TY.run_item(item, scen, O, in);
-            else T.run_item(item, scen, O, in);
+            if (yf) TY.run_item(item, scen, O, in, bnd);
+            else T.run_item(item, scen, O, in, bnd);
         }
         if (!grid_sync(reinterpret_cast<unsigned long long*>(B.ctl + 2), arrivals, a.wait_cycles, a.err)) break;
     }

@@ -354,7 +354,7 @@ struct cliffs_grid {
     int kind = 0;                            // 0 fused 2D, 1 x only, 2 y only
     int S = 32, nstrips = 0, nseg = 0;
     std::vector<unsigned char> hard;         // [nstrips][ny]: dry nodes in the strip's window within 3 rows
-    std::vector<double> strip_cost;          // per strip: the cost of its rows (item_cost)
+    std::vector<int> strip_slow;             // per strip: how many such rows
     ItemSet march, tile;                     // work items of the fused kernel (1D: samples only) and of the tiles
     ItemSet batch;                           // and of the persistent run by marching warps, made when first needed
     int tile_R = 0, tile_rows = 0;           // rows per tile in open water; the largest tile with its halo
@@ -518,27 +518,29 @@ int build_samples(cliffs_grid* g, ItemSet& set) {
     return CLIFFS_OK;
 }
 
-// Work items of the fused kernel. A row whose window has dry nodes within three rows takes the
-// general path, which costs about SLOW_COST rows of open water; every strip is cut into as
-// many segments as its cost holds S rows of open water, at equal costs, so that the warps of
-// one launch take about the same time. (With strips cut into equal numbers of rows, the warps
-// that cross an island decided the time of the launch: 157 us on a 4096^2 grid with ten
-// islands whose rows outside the islands' windows alone take 121 us.)
-const double SLOW_COST = 2.5;
+// Work items of the step kernels. A row whose window has dry nodes within three rows takes the
+// general path, which costs a marching warp about MARCH_SLOW rows of open water and a tile
+// about TILE_SLOW; every strip is cut into as many segments as its cost holds S rows of open
+// water, at equal costs, so that the items of one launch take about the same time. (With
+// strips cut into equal numbers of rows, the warps that cross an island decided the time of
+// the launch: 157 us on a 4096^2 grid with ten islands whose open-water rows alone take 121.) Measured at
+// MARCH_SLOW 2, 2.5, 3, 3.5: 2048^2 geographic 53.9, 51.7, 49.2, 50.5 us per step, 48 scenarios of
+// 512^2 106, 95.6, 94.2, 98.6. By tiles at TILE_SLOW 2, 2.5: 1201 x 901 24.8 and 26.3 us per step, but a
+// 331 x 287 nested child 1.38 and 1.18 ms per 120 steps and 300 x 257 1.94 and 1.84 ms per 200.
+const double MARCH_SLOW = 3.0, TILE_SLOW = 2.5;
 
-double strip_row_cost(const cliffs_grid* g, int st, int r) {
-    return g->hard[(size_t)st * g->ny + r] ? SLOW_COST : 1.0;
-}
+double strip_cost(const cliffs_grid* g, int st, double slow) { return g->ny + (slow - 1.0) * g->strip_slow[st]; }
 
-void cut_items(const cliffs_grid* g, int S, std::vector<int4>& items) {
+void cut_items(const cliffs_grid* g, int S, double slow, std::vector<int4>& items) {
     items.clear();
     for (int st = 0; st < g->nstrips; ++st) {
-        const double cost = g->strip_cost[st];
+        const double cost = strip_cost(g, st, slow);
+        const unsigned char* hard = g->hard.data() + (size_t)st * g->ny;
         const int nseg = std::max(1, std::min(g->ny, (int)std::ceil(cost / S - 1e-9)));
         double sum = 0.0;
         int r0 = 0, cut = 1;
         for (int r = 0; r < g->ny; ++r) {
-            sum += strip_row_cost(g, st, r);
+            sum += hard[r] ? slow : 1.0;
             if (r + 1 == g->ny || (cut < nseg && sum >= cost * cut / nseg - 1e-9)) {
                 items.push_back(make_int4(st, r0, r + 1, 0));
                 r0 = r + 1;
@@ -560,12 +562,12 @@ int set_rows_per_warp(cliffs_grid* g, int S) {
     g->S = S;
     g->nseg = (g->ny + S - 1) / S;
     if (g->kind != 0) return build_samples(g, g->march);
-    cut_items(g, S, g->march.items);
+    cut_items(g, S, MARCH_SLOW, g->march.items);
     return upload_items(g, g->march);
 }
 
 int set_tile_rows(cliffs_grid* g, int R) {
-    cut_items(g, R, g->tile.items);
+    cut_items(g, R, TILE_SLOW, g->tile.items);
     g->tile_R = R;
     g->tile_rows = 0;
     for (const int4& it : g->tile.items) g->tile_rows = std::max(g->tile_rows, it.z - it.y + 6);
@@ -573,10 +575,10 @@ int set_tile_rows(cliffs_grid* g, int R) {
 }
 
 // warps of one fused launch with S rows per warp, and the warps resident at once
-long long fused_warps(const cliffs_grid* g, int S) {
+long long fused_warps(const cliffs_grid* g, int S, double slow = MARCH_SLOW) {
     long long n = 0;
     for (int st = 0; st < g->nstrips; ++st)
-        n += std::max(1, std::min(g->ny, (int)std::ceil(g->strip_cost[st] / S - 1e-9)));
+        n += std::max(1, std::min(g->ny, (int)std::ceil(strip_cost(g, st, slow) / S - 1e-9)));
     return n * g->B;
 }
 
@@ -601,17 +603,16 @@ int wave_rows(const cliffs_grid* g, int waves) {
 // Modelled time of a launch of n warps with S rows each, in units of the time a scheduler
 // with its four warps takes per row (0.81 us on the 8192^2 grid): a warp takes S rows and
 // about 3.7 more (rows above and below its own, the first copies); full waves take 1 per row,
-// a last wave of one to four warps per scheduler 0.62, 0.74, 0.86 or 1. Launches a little
-// over full waves find room beside warps that end early (3 %). Against measured times over S on grids
-// of 200^2 to 8192^2 the model's choice is within 5 % of the best (8192^2: 435 us at S = 32,
-// 425 at 64, 429 at 128, 483 at 16; 1024^2: 22.9 at 10, 25.1 at 16, 27.1 at 8; 2048^2
-// geographic: 59.3 at 40, 63.8 at 20, 73.0 at 32).
+// a last wave of one to four warps per scheduler 0.62, 0.74, 0.86 or 1, and a twelfth of a wave
+// is lost to warps that take longer than the rest. Measured over S: 8192^2 435 us at 32, 425
+// at 64, 429 at 128, 483 at 16; 4096^2 128 at 32, 127 at 64 and 128 but 154 at 192 (a few warps past
+// one wave of long items cost another wave); 2048^2 geographic 59.3 at 40, 63.8 at 20, 73.0 at 32.
 double launch_cost(int S, long long n, long long resident, long long nsched) {
     const double last[5] = {0.0, 0.62, 0.74, 0.86, 1.0};
-    const double x = 0.97 * (double)n / (double)resident;
+    const double x = (double)n / (double)resident;
     const double full = std::floor(x);
     const int q = std::min(4, (int)std::ceil((x - full) * (double)resident / (double)nsched));
-    return (S + 3.7) * (full + last[q]);
+    return (S + 3.7) * (full + last[q] + 0.08);
 }
 
 // Rows per tile: the smallest modelled time of a launch of the tile kernel. A block's time is
@@ -623,7 +624,7 @@ int choose_tile(cliffs_grid* g) {
     double best = 1e300;
     int bestR = rmax;
     for (int R = 1; R <= rmax; ++R) {
-        const long long n = fused_warps(g, R);
+        const long long n = fused_warps(g, R, TILE_SLOW);
         const long long rounds = (n + resident - 1) / resident;
         // one block alone on an SM runs faster than two
         const double share = rounds == 1 && 2 * n <= resident ? 0.6 : 1.0;
@@ -657,7 +658,7 @@ int choose_batch(cliffs_grid* g) {
             cost += (double)((n1 * ((g->B * q + 3) / 4) + resident - 1) / resident) * (S + 3.7);
         if (cost < best) { best = cost; bestS = S; }
     }
-    cut_items(g, bestS, g->batch.items);
+    cut_items(g, bestS, MARCH_SLOW, g->batch.items);
     return upload_items(g, g->batch);
 }
 
@@ -1214,9 +1215,9 @@ int cliffs_set_bathy(cliffs_grid* g, const double* x, const double* y, const dou
                 else if (last - r <= 3) h[r] = 2;
             }
         }
-        g->strip_cost.assign(nstrips, 0.0);
+        g->strip_slow.assign(nstrips, 0);
         for (int st = 0; st < nstrips; ++st)
-            for (int r = 0; r < ny; ++r) g->strip_cost[st] += strip_row_cost(g, st, r);
+            for (int r = 0; r < ny; ++r) g->strip_slow[st] += g->hard[(size_t)st * ny + r] != 0;
     }
     int rc = choose_geometry(g);
     if (rc) return rc;
@@ -1894,7 +1895,7 @@ static int adjoint_core(cliffs_grid* g, int scenario, int64_t n, int32_t checkpo
         int Sr = 16;
         while (Sr < ny && fused_warps(g, Sr) / g->B * NG > cap) Sr += 2;
         if (Sr != g->adj_S || g->adj_items.empty()) {
-            cut_items(g, Sr, g->adj_items);
+            cut_items(g, Sr, MARCH_SLOW, g->adj_items);
             cudaFree(g->adj_items_dev);
             g->adj_items_dev = nullptr;
             CK(cudaMalloc(&g->adj_items_dev, sizeof(int4) * g->adj_items.size()));

@@ -461,7 +461,7 @@ struct FusedWarp {
         float* po = out_row(k - 2);
         while (true) {
             if (q == SLOT_ROWS) {
-                if (!next_slot(k, __all_sync(FULL, sw))) return false;
+                if (!next_slot(k, __all_sync(FULL, sw) && k < kgen)) return false;
                 q = 0;
                 s = at(cs, 0);
             }

@@ -57,6 +57,24 @@ def test_tiles_equal_marching_warps(nx, ny, kw):
         _same(outs[0], o)
 
 
+@pytest.mark.parametrize("kw", [dict(solver=1), dict(open_edges=8), dict(open_edges=4, alternate=1), dict()])
+@pytest.mark.parametrize("ny", [11, 18])
+def test_every_item_height_gives_the_same_bits(ny, kw):
+    """Items of 1 to ny rows (cut unequally beside dry nodes): the last rows of an item at, just
+    below and just above the grid's last row, and at the edges of the four-row slots."""
+    g, eta = _grid(90, ny, **kw)
+    outs = []
+    for rows in [None, *range(1, ny + 1)]:
+        if rows:
+            g.set_rows_per_warp(rows)
+        g.set_initial(eta)
+        g.step(6)
+        outs.append(_result(g))
+    g.close()
+    for o in outs[1:]:
+        _same(outs[0], o)
+
+
 def test_batch_with_durations_by_tiles_equals_marching_warps():
     durations = np.array([11, 4, 0, 17, 9], np.int64)
     outs = []

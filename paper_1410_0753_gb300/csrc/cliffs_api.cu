@@ -358,7 +358,7 @@ struct cliffs_grid {
     ItemSet march, tile;                     // work items of the fused kernel (1D: samples only) and of the tiles
     ItemSet batch;                           // and of the persistent run by marching warps, made when first needed
     int tile_R = 0, tile_rows = 0;           // rows per tile in open water; the largest tile with its halo
-    bool S_set = false;                      // S was set or tuned by the caller: steps march
+    int S_set = 0;                           // S was tuned (1) or set (2) by the caller: steps march
     // timing
     bool timing = false;
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev;
@@ -688,7 +688,7 @@ int choose_geometry(cliffs_grid* g) {
         }
         const int rc = set_rows_per_warp(g, bestS);
         if (rc) return rc;
-        g->S_set = false;
+        g->S_set = 0;
         g->batch.items.clear();
         return choose_tile(g);
     }
@@ -1600,11 +1600,11 @@ int cliffs_run_persistent(cliffs_grid* g, int64_t n) {
     }
     // no more blocks than the batch has work (each one more makes the barrier slower)
     const bool tiles = by_tiles(g);
-    if (!tiles && !g->S_set && g->batch.items.empty()) {
+    if (!tiles && g->S_set < 2 && g->batch.items.empty()) {
         rc = choose_batch(g);
         if (rc) return rc;
     }
-    const ItemSet& set = tiles ? g->tile : g->S_set ? g->march : g->batch;
+    const ItemSet& set = tiles ? g->tile : g->S_set == 2 ? g->march : g->batch;
     const long long per = tiles ? 1 : fused_warps_per_block();
     const long long work = ((long long)set.items.size() * g->B + per - 1) / per;
     const int blocks = (int)std::min<long long>(tiles ? g->pblocks_tile : g->pblocks, work);
@@ -2201,7 +2201,7 @@ int cliffs_set_rows_per_warp(cliffs_grid* g, int32_t rows) {
     if (!g->have_bathy) return set_err(CLIFFS_ERR_STATE, "set_bathy first (it chooses the geometry)");
     if (g->kind != 0) return set_err(CLIFFS_ERR_ARG, "a 1D grid has no tile shape");
     if (rows < 1 || rows > 8192) return set_err(CLIFFS_ERR_ARG, "rows per warp %d outside 1..8192", rows);
-    g->S_set = true;
+    g->S_set = 2;
     return set_rows_per_warp(g, rows);
 }
 
@@ -2245,24 +2245,39 @@ int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     int rc = CLIFFS_OK;
+    float tbest = 1e30f;                               // of the trials of one candidate, ms
+    auto trial = [&](bool by_tile) -> int {
+        tbest = 1e30f;
+        for (int t = 0; t <= trials; ++t) {             // the first launch warms up
+            cudaMemsetAsync(flush, t & 0xff, flush_bytes, s);
+            cudaEventRecord(e0, s);
+            const cudaError_t le = by_tile ? launch_step_tile(a, g->B, s) : launch_step_fused(a, g->maps[cur], g->B, s);
+            cudaEventRecord(e1, s);
+            if (le != cudaSuccess) return set_err(CLIFFS_ERR_CUDA, "autotune launch: %s", cudaGetErrorString(le));
+            if (cudaEventSynchronize(e1) != cudaSuccess) return set_err(CLIFFS_ERR_CUDA, "autotune sync");
+            float ms = 0.f;
+            cudaEventElapsedTime(&ms, e0, e1);
+            if (t > 0) tbest = std::min(tbest, ms);
+        }
+        return CLIFFS_OK;
+    };
+    // a grid small enough to step by tiles keeps doing so unless some rows per warp are faster
+    g->S_set = 0;
+    const bool tiles = by_tiles(g);
+    double tile_ms = 1e30;
+    if (tiles) {
+        use_items(g->tile, a);
+        rc = trial(true);
+        tile_ms = tbest;
+    }
+    if (rc) list.clear();
     for (int S : list) {
         if (S > 2 * g->ny && S != list[0]) break;
         rc = set_rows_per_warp(g, S);
         if (rc) break;
         a.S = g->S; a.nseg = g->nseg; a.samp_ptr = g->march.samp_ptr; a.samp = g->march.samp;
         a.items = g->march.dev; a.nitems = (int)g->march.items.size();
-        float tbest = 1e30f;
-        for (int t = 0; t <= trials; ++t) {             // the first launch warms up
-            cudaMemsetAsync(flush, t & 0xff, flush_bytes, s);
-            cudaEventRecord(e0, s);
-            cudaError_t le = launch_step_fused(a, g->maps[cur], g->B, s);
-            cudaEventRecord(e1, s);
-            if (le != cudaSuccess) { rc = set_err(CLIFFS_ERR_CUDA, "autotune launch: %s", cudaGetErrorString(le)); break; }
-            if (cudaEventSynchronize(e1) != cudaSuccess) { rc = set_err(CLIFFS_ERR_CUDA, "autotune sync"); break; }
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (t > 0) tbest = std::min(tbest, ms);
-        }
+        rc = trial(false);
         if (rc) break;
         if (cand) cand[n] = S;
         if (us) us[n] = 1e3 * tbest;
@@ -2276,7 +2291,7 @@ int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32
     cudaMemcpy(h, g->err, sizeof(h), cudaMemcpyDeviceToHost);
     cudaMemset(g->err, 0, sizeof(h));
     const int rc2 = set_rows_per_warp(g, rc ? oldS : bestS);
-    g->S_set = !rc && !rc2;
+    g->S_set = !rc && !rc2 && best < tile_ms ? 1 : 0;
     if (ncand) *ncand = n;
     if (rc) return rc;
     if (rc2) return rc2;

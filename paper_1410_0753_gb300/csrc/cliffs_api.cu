@@ -1466,12 +1466,27 @@ int cliffs_step_n(cliffs_grid* g, int64_t n) {
     // A run recorded with every state kept (checkpoint j is the state after j steps, laid out as
     // a state buffer): the tile kernel steps from checkpoint to checkpoint, and the last one is
     // copied back at the end, in place of a copy of every state (6 of 26 us per step of a 1024^2 grid).
+    // The first step of a call reads the state buffer itself: the caller may have written into it
+    // since the state was recorded (cliffs_state_ptrs).
     const bool in_record = tiles && g->rec_K == 1 && !g->bnd_any && g->limit_h.empty();
     if (in_record) {
         rc = grow_checkpoints(g, last);
         if (rc) return rc;
     }
     const size_t rec_state = (size_t)3 * g->B * g->plane;
+    // the state goes back into its buffer however the call ends (a failed launch included)
+    struct CopyBack {
+        cliffs_grid* g;
+        size_t n;
+        long long from;              // steps done when the call began; -1: nothing to copy
+        cudaError_t run() {
+            const bool due = from >= 0 && g->step > from;
+            from = -1;
+            return !due ? cudaSuccess : cudaMemcpyAsync(g->st[g->step & 1], g->rec_ckpt + n * g->step, sizeof(float) * n,
+                                                        cudaMemcpyDeviceToDevice, g->stream);
+        }
+        ~CopyBack() { run(); }
+    } back{g, rec_state, in_record ? g->step : -1};
     const double t_end = g->bnd_any ? bnd_end(g) : 1e300;
     // 1D lines: all the steps in one launch (at most LINE_STEPS, some tens of milliseconds),
     // except one step alone, lines too long for a block, boundary input, timed launches and the
@@ -1534,7 +1549,7 @@ int cliffs_step_n(cliffs_grid* g, int64_t n) {
         if (tiles) {
             use_items(g->tile, a);
             if (in_record) {
-                a.eta_in = g->rec_ckpt + rec_state * (st - 1);
+                if (k > 0) a.eta_in = g->rec_ckpt + rec_state * (st - 1);
                 a.eta_out = g->rec_ckpt + rec_state * st;
             }
             le = launch_step_tile(a, g->B, s);
@@ -1556,9 +1571,7 @@ int cliffs_step_n(cliffs_grid* g, int64_t n) {
             }
         }
     }
-    if (in_record)
-        CK(cudaMemcpyAsync(g->st[g->step & 1], g->rec_ckpt + rec_state * g->step, sizeof(float) * rec_state,
-                           cudaMemcpyDeviceToDevice, s));
+    CK(back.run());
     int h[4] = {0, 0, 0, 0};
     CK(cudaMemcpyAsync(h, g->err, sizeof(int) * 4, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

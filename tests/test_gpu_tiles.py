@@ -105,3 +105,28 @@ def test_line_in_one_launch_equals_a_launch_per_step(n, along_y, kw):
         g.close()
     assert np.isfinite(outs[0][0]).all()
     _same(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("every", [1, 3])
+@pytest.mark.parametrize("march", [0, 1])
+def test_recorded_run_takes_writes_through_the_state_views(march, every):
+    """What is written into the state views before the first step and between calls is what the
+    next step starts from, recorded or not."""
+    outs = []
+    for record in (0, 1):
+        g, eta = _grid(130, 70)
+        if march:
+            g.set_rows_per_warp(9)
+        g.set_initial(eta)
+        if record:
+            g.adjoint_record(every)
+        g.state_views()[1].fill_(0.125)
+        g.step(5)
+        for f, s in zip(g.state_views(), (0.5, 0.25, -1.0)):
+            f.mul_(s)
+        g.step(4)
+        g.state_views()[2].add_(0.0625)
+        g.step(1)
+        outs.append(_result(g))
+        g.close()
+    _same(outs[0], outs[1])

@@ -10,6 +10,7 @@ namespace cliffs {
 
 constexpr int LINE_PAD = 4;                        // nodes a window starts before its outputs
 constexpr int LINE_ARRAYS = 12;
+constexpr int LINE_MAX_SMEM = 227 * 1024;          // of one block
 
 static int line_floats(int n) { return (n + XOUT - 1) / XOUT * XOUT + 2 * LINE_PAD; }
 
@@ -106,7 +107,7 @@ k_line(const __grid_constant__ StepArgs a, const __grid_constant__ BatchArgs B, 
     if (bad) atomicOr(a.err, ERRF_NONFINITE);
 }
 
-bool line_fits(int nodes) { return (size_t)line_floats(nodes) * LINE_ARRAYS * 4 <= 227u * 1024u; }
+bool line_fits(int nodes) { return (size_t)line_floats(nodes) * LINE_ARRAYS * 4 <= (size_t)LINE_MAX_SMEM; }
 
 cudaError_t launch_line(const StepArgs& a, const BatchArgs& b, int batch, long long step0, long long n, int nsamp,
                         int along_y, cudaStream_t s) {
@@ -116,7 +117,9 @@ cudaError_t launch_line(const StepArgs& a, const BatchArgs& b, int batch, long l
                                      (const void*)k_line<false, true, true>, (const void*)k_line<true, true, true>};
     const int N = along_y ? a.ny : a.nx, smem = line_floats(N) * LINE_ARRAYS * 4;
     const void* k = t[(a.K.fric ? 1 : 0) + (a.K.inv_dt2 > 0.f ? 2 : 0) + (a.open_edges ? 4 : 0)];
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // always the maximum, not this line's size: the attribute belongs to the kernel, and another
+    // thread may launch it for a longer line between these two calls
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, LINE_MAX_SMEM);
     if (e != cudaSuccess) return e;
     StepArgs aa = a;
     BatchArgs bb = b;

@@ -3,10 +3,12 @@ launches they stand in for. All of them run the same arithmetic per node, so the
 equal bit for bit: state, max-wave and gauge records. Sizes at the edges of windows (64
 columns, 56 finished) and tiles, one row or column either side, down to the smallest grids.
 """
+import threading
+
 import numpy as np
 import pytest
 
-from paper_1410_0753_gb300 import CliffsGrid
+from paper_1410_0753_gb300 import CliffsError, CliffsGrid
 
 pytestmark = pytest.mark.gpu
 
@@ -130,3 +132,33 @@ def test_recorded_run_takes_writes_through_the_state_views(march, every):
         outs.append(_result(g))
         g.close()
     _same(outs[0], outs[1])
+
+
+def test_lines_of_different_lengths_on_two_threads():
+    """A long and a short line, each on its own thread, share the kernel and must not change what
+    the other's launch may ask for (distinct handles may be used from distinct threads)."""
+    grids, want, errors = [], [], []
+    for n in (4000, 60):
+        g, eta = _grid(n, 1)
+        g.set_initial(eta)
+        g.step(20000)
+        want.append(_result(g))
+        g.set_initial(eta)
+        grids.append(g)
+
+    def run(g):
+        try:
+            for _ in range(2000):
+                g.step(10)
+        except CliffsError as e:
+            errors.append(str(e))
+
+    threads = [threading.Thread(target=run, args=(g,)) for g in grids]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors
+    for g, w in zip(grids, want):
+        _same(_result(g), w)
+        g.close()

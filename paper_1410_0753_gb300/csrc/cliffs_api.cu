@@ -22,6 +22,7 @@
 #include "internal.h"
 #include "adjoint.h"
 #include "filter.cuh"
+#include "pointers.h"
 #include "sweep.cuh"
 
 using namespace cliffs;
@@ -427,14 +428,6 @@ struct cliffs_grid {
 };
 
 namespace {
-
-// whether p is memory of the current device (kernels may read it), rather than host or managed
-bool on_device(const void* p) {
-    cudaPointerAttributes at;
-    int dev = -1;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return false; }
-    return at.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess && at.device == dev;
-}
 
 int ensure_tmp(cliffs_grid* g, size_t bytes) {
     if (bytes <= g->tmp_bytes) return CLIFFS_OK;
@@ -1267,8 +1260,8 @@ int cliffs_set_initial(cliffs_grid* g, int scenario, const float* eta, const flo
                                                         g->pitch, g->cfg.h_min, dwall);
         CK(cudaGetLastError());
     }
-    // fields in device memory are read where they are; anything else is copied into the planes
-    const bool direct = !quake && on_device(eta) && (!u || on_device(u)) && (!v || on_device(v));
+    // fields a kernel may read are read where they are; anything else is copied into the planes
+    const bool direct = !quake && kernel_may_read(eta) && (!u || kernel_may_read(u)) && (!v || kernel_may_read(v));
     if (!direct) {
         if (!quake) CK(cudaMemcpy2DAsync(g->eta[0] + off, pitchb, eta, rowb, rowb, rows, cudaMemcpyDefault, s));
         if (u) CK(cudaMemcpy2DAsync(g->u[0] + off, pitchb, u, rowb, rowb, rows, cudaMemcpyDefault, s));

@@ -11,6 +11,7 @@
 #include "cliffs.h"
 #include "filter.cuh"
 #include "internal.h"
+#include "pointers.h"
 
 namespace {
 
@@ -102,7 +103,7 @@ int cliffs_depth_filter_noalloc(const double* depth, double* out, int32_t nx, in
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const unsigned blocks = (unsigned)((N + 255) / 256);
     const double* src = depth;
-    if (out != depth && ti != cudaMemoryTypeDevice && ti != cudaMemoryTypeManaged) {
+    if (out != depth && !cliffs::kernel_may_read(depth)) {
         e = cudaMemcpyAsync(out, depth, sizeof(double) * N, cudaMemcpyDefault, s);
         if (e != cudaSuccess) return fail(CLIFFS_ERR_CUDA, "copy of the input depth", e);
         src = out;

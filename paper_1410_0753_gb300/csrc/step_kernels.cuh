@@ -106,10 +106,11 @@ __device__ __forceinline__ int open_end_y(const StepArgs& a, int row) {
 __device__ __forceinline__ int runaway(float e, float u, float v) {
     return !(fabsf(e) + fabsf(u) + fabsf(v) < 3e5f);
 }
-// The same test accumulated branch-free over the rows of a warp's work: the sum of
-// e^2 + u^2 + v^2 over its stored nodes reaches 9e10 when any node reaches 3e5 in a component
-// (no physical state sums that high over a warp's few thousand nodes), and a non-finite
-// value makes it non-finite.
+// The same test accumulated branch-free over the rows of one work item: the sum of e^2 + u^2 +
+// v^2 over a lane's stored nodes reaches 9e10 when any node reaches 3e5 in a component, and a
+// non-finite value makes it non-finite. No physical state sums that high over an item's rows
+// (land far above the sea counts with its eta = -d; over the steps of a persistent run it
+// would), so the sum is tested and cleared after every item.
 constexpr float RUNAWAY_SQ = 9e10f;
 
 // What changes from one step to the next: the input state's TMA descriptors, the output
@@ -595,12 +596,14 @@ struct FusedWarp {
             bad |= 2;
             return false;
         }
+        bad |= !(chk_out.x + chk_out.y < RUNAWAY_SQ);
+        chk_out = v2(0.f);
         write_samples(a, O, idx, b, lane);
         return true;
     }
 
     __device__ __forceinline__ void report() {
-        bad |= !(chk_x.x + chk_x.y == 0.f) | !(chk_out.x + chk_out.y < RUNAWAY_SQ);
+        bad |= !(chk_x.x + chk_x.y == 0.f);
         if (bad) atomicOr(a.err, (bad & 2) ? (ERRF_TIMEOUT | ERRF_NONFINITE) : ERRF_NONFINITE);
     }
 };

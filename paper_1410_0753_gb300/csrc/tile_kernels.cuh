@@ -262,6 +262,8 @@ struct Tile {
         sweep_rows();
         __syncthreads();
         sweep_cols();
+        bad |= !(chk_out.x + chk_out.y < RUNAWAY_SQ);
+        chk_out = v2(0.f);
         if (a.samp_ptr && (O.rec_g || O.rec_n)) {
             __syncthreads();                          // the whole tile is stored
             if (wib == 0) write_samples(a, O, idx, b, lane);
@@ -269,7 +271,7 @@ struct Tile {
     }
 
     __device__ __forceinline__ void report() {
-        bad |= !(chk_x.x + chk_x.y == 0.f) | !(chk_out.x + chk_out.y < RUNAWAY_SQ);
+        bad |= !(chk_x.x + chk_x.y == 0.f);
         if (bad) atomicOr(a.err, ERRF_NONFINITE);
     }
 };

@@ -162,3 +162,30 @@ def test_lines_of_different_lengths_on_two_threads():
     for g, w in zip(grids, want):
         _same(_result(g), w)
         g.close()
+
+
+def _high_land(nx, ny, top):
+    """A shallow bay beside land `top` metres high, whose dry nodes carry eta = -d."""
+    d = np.full((ny, nx), 20.0)
+    d[:, nx // 2:] = -top
+    g = CliffsGrid(nx, ny, 1.0, gauges=[(3, 3)], maxout=7)
+    g.set_bathy(50.0 * np.arange(nx), 50.0 * np.arange(ny), d, False)
+    eta = np.where(d > 0, 0.0, -d).astype(np.float32)
+    eta[:, :6] = 0.25
+    return g, eta
+
+
+@pytest.mark.parametrize("march", [0, 1])
+def test_long_persistent_run_beside_high_land(march):
+    """The runaway test of a persistent run looks at one step at a time, as a launch per step does:
+    high dry land does not add up over the steps."""
+    outs = []
+    for persistent in (False, True):
+        g, eta = _high_land(70, 60, 5000.0)
+        if march:
+            g.set_rows_per_warp(20)
+        g.set_initial(eta)
+        g.step(3000, persistent=persistent)
+        outs.append(_result(g))
+        g.close()
+    _same(outs[0], outs[1])

@@ -522,10 +522,15 @@ int build_samples(cliffs_grid* g, ItemSet& set) {
 // 331 x 287 nested child 1.38 and 1.18 ms per 120 steps and 300 x 257 1.94 and 1.84 ms per 200.
 const double MARCH_SLOW = 3.0, TILE_SLOW = 2.5;
 
+// Rows of an item at most, whatever the caller asks for: the runaway test (RUNAWAY_SQ) sums eta^2
+// over a lane's two columns of the item, where land 9300 m high stays below its bound on 512 rows.
+const int ITEM_ROWS = 512;
+
 double strip_cost(const cliffs_grid* g, int st, double slow) { return g->ny + (slow - 1.0) * g->strip_slow[st]; }
 
 void cut_items(const cliffs_grid* g, int S, double slow, std::vector<int4>& items) {
     items.clear();
+    S = std::min(S, ITEM_ROWS);
     for (int st = 0; st < g->nstrips; ++st) {
         const double cost = strip_cost(g, st, slow);
         const unsigned char* hard = g->hard.data() + (size_t)st * g->ny;
@@ -570,6 +575,7 @@ int set_tile_rows(cliffs_grid* g, int R) {
 // warps of one fused launch with S rows per warp, and the warps resident at once
 long long fused_warps(const cliffs_grid* g, int S, double slow = MARCH_SLOW) {
     long long n = 0;
+    S = std::min(S, ITEM_ROWS);
     for (int st = 0; st < g->nstrips; ++st)
         n += std::max(1, std::min(g->ny, (int)std::ceil(strip_cost(g, st, slow) / S - 1e-9)));
     return n * g->B;

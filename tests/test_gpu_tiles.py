@@ -189,3 +189,16 @@ def test_long_persistent_run_beside_high_land(march):
         outs.append(_result(g))
         g.close()
     _same(outs[0], outs[1])
+
+
+def test_one_step_of_tall_items_beside_high_land():
+    """Rows per warp past what one runaway test may cover."""
+    outs = []
+    for rows in (16, 8192):
+        g, eta = _high_land(64, 2200, 8000.0)
+        g.set_rows_per_warp(rows)
+        g.set_initial(eta)
+        g.step(2)
+        outs.append(_result(g))
+        g.close()
+    _same(outs[0], outs[1])

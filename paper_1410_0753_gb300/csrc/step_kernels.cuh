@@ -253,9 +253,12 @@ struct FusedWarp {
     __device__ __forceinline__ const float* at(int s, int q) const { return ring + s * a.slot_floats + q * XWIN; }
 
     // one lane starts the boxes of the item's next slot (rows k0 + 4 nfill ..; the max-wave
-    // rows two rows behind, where the open-water path emits)
+    // rows two rows behind, where the open-water path emits). The caller has the warp meet first:
+    // the slot may hold a row that other lanes have just read. The fence orders those reads (the
+    // generic proxy) before the copy's writes (the async proxy).
     __device__ __forceinline__ void fill() {
         if (lane == 0) {
+            fence_proxy_async();
             float* dst = ring + head * a.slot_floats;
             const int row = k0 + SLOT_ROWS * nfill;
             mbar_arrive_tx(&bar[head], tx);
@@ -543,6 +546,7 @@ struct FusedWarp {
         nfill = nread = 0;
         cs = head;
         const int first = head;
+        __syncwarp();                              // the item before is done with the ring
         while (nfill < min(a.nslots, ntot)) fill();
         ym.init();
         // An open first or last row and eq. (solver1)'s flux around one take the general path: no

@@ -202,3 +202,18 @@ def test_one_step_of_tall_items_beside_high_land():
         outs.append(_result(g))
         g.close()
     _same(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(alternate=1)])
+def test_warps_that_take_several_items_a_step(kw):
+    """More items than the GPU holds warps: a marching warp of the persistent run goes from one
+    item's last ring slot to the next one's first within a step."""
+    batch, outs = 24, []
+    for persistent in (False, True):
+        g, eta = _grid(130, 70, batch=batch, **kw)
+        g.set_rows_per_warp(1)
+        g.set_initial(np.stack([eta * (0.2 + 0.05 * b) for b in range(batch)]))
+        g.step(12, persistent=persistent)
+        outs.append([r for b in range(batch) for r in _result(g, b)])
+        g.close()
+    _same(outs[0], outs[1])

@@ -278,7 +278,7 @@ int cliffs_adjoint_velocity(cliffs_grid* g, float* dL_du0, float* dL_dv0);
  * longer warps, and the count of warps against the resident slots decides the tail). Each
  * candidate S is timed over `trials` launches (after one warm-up) that read the current
  * state and write scratch planes, with max-wave and records off, each after a 192 MiB write
- * that evicts the inputs from L2; the fastest is kept for later steps. (A grid small enough that the
+ * that evicts the inputs from L2; the fastest is kept for later steps, the persistent run's included. (A grid small enough that the
  * library steps it by tiles of its own choice keeps those when they are faster than every
  * candidate.) The grid's state, maxima and records are unchanged.
  * Optional outputs: cand[] and us[] (capacity 16) receive the candidates and their best

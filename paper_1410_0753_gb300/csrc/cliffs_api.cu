@@ -359,7 +359,7 @@ struct cliffs_grid {
     ItemSet march, tile;                     // work items of the fused kernel (1D: samples only) and of the tiles
     ItemSet batch;                           // and of the persistent run by marching warps, made when first needed
     int tile_R = 0, tile_rows = 0;           // rows per tile in open water; the largest tile with its halo
-    int S_set = 0;                           // S was tuned (1) or set (2) by the caller: steps march
+    bool S_set = false;                      // S was set or tuned by the caller: steps march
     // timing
     bool timing = false;
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev;
@@ -641,11 +641,13 @@ bool by_tiles(const cliffs_grid* g) {
     return g->kind == 0 && !g->S_set && (long long)g->tile.items.size() * g->B <= 2ll * num_sms();
 }
 
-// Rows per warp of the persistent run by marching warps: its items are handed out in rounds of
-// the resident warps, so the smallest sum of rounds * (rows + 3.7) counts, over batches that
-// shrink as scenarios end (all of them running, three quarters, half, a quarter). 48 scenarios
-// of 512^2, all running: 95.5 us per step at 28 rows, 109 at 24, 103 at 40, 131 at 20 (the choice
-// for one launch per step).
+// Rows per warp of the persistent run by marching warps when the caller neither set nor tuned them:
+// its items are handed out in rounds of the resident warps, so the smallest sum of rounds * (rows
+// + 3.7) counts, over batches that shrink as scenarios end (all of them running, three quarters,
+// half, a quarter). That takes items to cost the same; those with a shore cost more, and a warp
+// may draw the same kind in every round. Rows tuned by a launch per step do better: 512^2,
+// uneven durations, 256 scenarios 94.4 Gcell-updates/s by this rule and 101.8 tuned, 128 89.5 and
+// 98.6, 64 74.4 and 83 +- 2, 20 63.1 and 69 +- 2, but 48 87.4 and 83.4.
 int choose_batch(cliffs_grid* g) {
     const long long resident = resident_warps(g);
     double best = 1e300;
@@ -687,7 +689,7 @@ int choose_geometry(cliffs_grid* g) {
         }
         const int rc = set_rows_per_warp(g, bestS);
         if (rc) return rc;
-        g->S_set = 0;
+        g->S_set = false;
         g->batch.items.clear();
         return choose_tile(g);
     }
@@ -1612,11 +1614,11 @@ int cliffs_run_persistent(cliffs_grid* g, int64_t n) {
     }
     // no more blocks than the batch has work (each one more makes the barrier slower)
     const bool tiles = by_tiles(g);
-    if (!tiles && g->S_set < 2 && g->batch.items.empty()) {
+    if (!tiles && !g->S_set && g->batch.items.empty()) {
         rc = choose_batch(g);
         if (rc) return rc;
     }
-    const ItemSet& set = tiles ? g->tile : g->S_set == 2 ? g->march : g->batch;
+    const ItemSet& set = tiles ? g->tile : g->S_set ? g->march : g->batch;
     const long long per = tiles ? 1 : fused_warps_per_block();
     const long long work = ((long long)set.items.size() * g->B + per - 1) / per;
     const int blocks = (int)std::min<long long>(tiles ? g->pblocks_tile : g->pblocks, work);
@@ -2213,7 +2215,7 @@ int cliffs_set_rows_per_warp(cliffs_grid* g, int32_t rows) {
     if (!g->have_bathy) return set_err(CLIFFS_ERR_STATE, "set_bathy first (it chooses the geometry)");
     if (g->kind != 0) return set_err(CLIFFS_ERR_ARG, "a 1D grid has no tile shape");
     if (rows < 1 || rows > 8192) return set_err(CLIFFS_ERR_ARG, "rows per warp %d outside 1..8192", rows);
-    g->S_set = 2;
+    g->S_set = true;
     return set_rows_per_warp(g, rows);
 }
 
@@ -2274,7 +2276,7 @@ int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32
         return CLIFFS_OK;
     };
     // a grid small enough to step by tiles keeps doing so unless some rows per warp are faster
-    g->S_set = 0;
+    g->S_set = false;
     const bool tiles = by_tiles(g);
     double tile_ms = 1e30;
     if (tiles) {
@@ -2303,7 +2305,7 @@ int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32
     cudaMemcpy(h, g->err, sizeof(h), cudaMemcpyDeviceToHost);
     cudaMemset(g->err, 0, sizeof(h));
     const int rc2 = set_rows_per_warp(g, rc ? oldS : bestS);
-    g->S_set = !rc && !rc2 && best < tile_ms ? 1 : 0;
+    g->S_set = !rc && !rc2 && best < tile_ms;
     if (ncand) *ncand = n;
     if (rc) return rc;
     if (rc2) return rc2;

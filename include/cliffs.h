@@ -277,8 +277,9 @@ int cliffs_adjoint_velocity(cliffs_grid* g, float* dL_du0, float* dL_dv0);
  * fused step owns: a warp walks S + 6 rows, so larger S means less halo work but fewer,
  * longer warps, and the count of warps against the resident slots decides the tail). Each
  * candidate S is timed over `trials` launches (after one warm-up) that read the current
- * state and write scratch planes, with max-wave and records off, each after a 192 MiB write
- * that evicts the inputs from L2; the fastest is kept for later steps, the persistent run's included. (A grid small enough that the
+ * state and write scratch planes, with max-wave and records off; where a step's planes do not fit
+ * in L2, each comes after a 192 MiB write that evicts its inputs, as the steps of a run do. The
+ * fastest is kept for later steps, the persistent run's included. (A grid small enough that the
  * library steps it by tiles of its own choice keeps those when they are faster than every
  * candidate.) The grid's state, maxima and records are unchanged.
  * Optional outputs: cand[] and us[] (capacity 16) receive the candidates and their best

@@ -2230,10 +2230,17 @@ int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32
     if (trials < 1) trials = 3;
     cudaStream_t s = g->stream;
     // scratch output planes: the trial steps read the current state and write elsewhere,
-    // with max-wave and records off, so the grid's state and outputs are untouched; before
-    // each trial a write larger than L2 evicts the inputs, as in a long run
+    // with max-wave and records off, so the grid's state and outputs are untouched. Where a
+    // step's planes (two states and the depth) exceed L2, a write larger than L2 evicts the
+    // inputs before each trial, as the steps of a run do; smaller grids find them in L2, as they do
+    // in a run (1024^2 with a shore: 27.5 us per step untuned, by tiles; with an eviction before each
+    // trial marching warps came out ahead, which take 30.1 in a run).
     const size_t pb = sizeof(float) * (size_t)g->B * g->plane;
-    const size_t flush_bytes = (size_t)192 << 20;
+    int dev = 0, l2 = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
+    const bool evict = 6 * pb + sizeof(float) * (size_t)g->plane > (size_t)l2;
+    const size_t flush_bytes = evict ? (size_t)192 << 20 : 0;
     float* scratch = nullptr;
     CK(cudaMalloc(&scratch, 3 * pb + flush_bytes));
     unsigned char* flush = reinterpret_cast<unsigned char*>(scratch + 3 * (pb / sizeof(float)));
@@ -2263,7 +2270,7 @@ int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32
     auto trial = [&](bool by_tile) -> int {
         tbest = 1e30f;
         for (int t = 0; t <= trials; ++t) {             // the first launch warms up
-            cudaMemsetAsync(flush, t & 0xff, flush_bytes, s);
+            if (evict) cudaMemsetAsync(flush, t & 0xff, flush_bytes, s);
             cudaEventRecord(e0, s);
             const cudaError_t le = by_tile ? launch_step_tile(a, g->B, s) : launch_step_fused(a, g->maps[cur], g->B, s);
             cudaEventRecord(e1, s);

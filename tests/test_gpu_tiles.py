@@ -247,3 +247,27 @@ def test_persistent_run_takes_the_tuned_rows():
     by_hand = best()
     g.close()
     assert abs(tuned - by_hand) <= 0.03 * by_hand, (tuned, by_hand, table)
+
+
+@pytest.mark.parametrize("n", [200, 512, 1024])
+def test_tuning_makes_no_small_grid_slower(n):
+    """The autotuner times under the conditions of a run: what it keeps for a grid whose step fits
+    in L2 is no slower than what the library chose (device time per step)."""
+    g, eta = _grid(n, n)
+
+    def best():
+        g.set_initial(eta)
+        times = []
+        for _ in range(6):
+            g.kernel_time(-1)
+            g.kernel_time(1)
+            g.step(100)
+            ms, launches = g.kernel_time(0)
+            times.append(ms / launches)
+        return min(times)
+
+    before = best()
+    table = g.autotune(3)
+    after = best()
+    g.close()
+    assert after <= 1.05 * before, (before, after, table)

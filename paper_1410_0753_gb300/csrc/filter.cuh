@@ -64,7 +64,9 @@ static __global__ void __launch_bounds__(256) k_filter_pass(const double* __rest
     __shared__ double T[FILTER_TILE + 2][FILTER_TILE];   // rows r0-1 .. r0+32 after the pass along x
     __shared__ short list[(FILTER_TILE + 2) * FILTER_TILE];
     __shared__ int count[2];
-    const int c0 = blockIdx.x * FILTER_TILE, r0 = blockIdx.y * FILTER_TILE;
+    // tiles are numbered along x first, in one grid dimension: a line along y has too many for the second
+    const unsigned across = (unsigned)(nx + FILTER_TILE - 1) / FILTER_TILE;
+    const int c0 = (int)(blockIdx.x % across) * FILTER_TILE, r0 = (int)(blockIdx.x / across) * FILTER_TILE;
     bool any = false;
     if (threadIdx.x < 2) count[threadIdx.x] = 0;
     __syncthreads();
@@ -115,7 +117,8 @@ static __global__ void __launch_bounds__(256) k_filter_pass(const double* __rest
 inline cudaError_t run_filter(double* d, double* tmp, int nx, int ny, double alpha, int* flags, cudaStream_t s,
                               int* passes) {
     cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(int) * FILTER_PASSES, s);
-    const dim3 grid((nx + FILTER_TILE - 1) / FILTER_TILE, (ny + FILTER_TILE - 1) / FILTER_TILE), block(256);
+    const dim3 grid((unsigned)((nx + FILTER_TILE - 1) / FILTER_TILE) * (unsigned)((ny + FILTER_TILE - 1) / FILTER_TILE));
+    const dim3 block(256);
     int h[FILTER_PASSES];
     const double a2 = alpha * alpha;
     const int e20 = std::ilogb(a2) << 20;

@@ -9,6 +9,7 @@ import time
 import numpy as np
 import pytest
 
+import oracle
 import workloads
 from paper_1410_0753_gb300 import CliffsError, CliffsGrid
 
@@ -271,3 +272,16 @@ def test_tuning_makes_no_small_grid_slower(n):
     after = best()
     g.close()
     assert after <= 1.05 * before, (before, after, table)
+
+
+def test_depth_filter_of_a_line_of_many_rows():
+    """A line along y of more nodes than 65535 tiles of rows hold, bit for bit the oracle's."""
+    n = 2_100_000
+    d = np.full((n, 1), 10.0)
+    d[1::50] = 100.0
+    g = CliffsGrid(1, n, 0.5)
+    g.set_bathy(np.zeros(1), 100.0 * np.arange(n), d, True)
+    got = g.depth()
+    g.close()
+    want, _ = oracle.depth_filter(d, 2.0, 0.1)
+    assert not np.array_equal(want, d) and np.array_equal(got, want)

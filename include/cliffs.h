@@ -381,7 +381,7 @@ int cliffs_kernel_time(cliffs_grid* g, int enable, double* ms, int64_t* launches
  * any stream capture. The kept address does not survive cudaDeviceReset. Every call on a
  * device shares the one array and leaves its last contents there (the flag is cleared
  * before each call): calls that overlap on the GPU (other streams or threads) race and give
- * wrong results. The call synchronises the stream once per group of passes (8, 16, 32, 44) to read
+ * wrong results. The call synchronises the stream once per group of passes (2, 4, 8, .. 38) to read
  * the flags. */
 #define CLIFFS_NOALLOC_MAX_CELLS (1 << 20)
 int cliffs_depth_filter_noalloc(const double* depth, double* out, int32_t nx, int32_t ny,

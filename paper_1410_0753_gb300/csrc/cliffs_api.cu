@@ -1076,7 +1076,7 @@ int cliffs_set_bathy(cliffs_grid* g, const double* x, const double* y, const dou
     cudaStream_t s = g->stream;
     CK(cudaMemcpyAsync(g->d64, depth, sizeof(double) * N, cudaMemcpyDefault, s));
     if (apply_filter) {
-        k_filter_raise<<<nblk(N), 256, 0, s>>>(g->d64, g->d64, N, min_depth);
+        k_filter_raise<<<nblk(N), 256, 0, s>>>(g->d64, g->d64, N, min_depth, reinterpret_cast<int*>(g->ured));
         CK(cudaGetLastError());
         int passes = 0;
         CK(run_filter(g->d64, g->d64b, nx, ny, alpha, reinterpret_cast<int*>(g->ured), s, &passes));

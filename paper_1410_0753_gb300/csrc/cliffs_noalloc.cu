@@ -108,7 +108,7 @@ int cliffs_depth_filter_noalloc(const double* depth, double* out, int32_t nx, in
         if (e != cudaSuccess) return fail(CLIFFS_ERR_CUDA, "copy of the input depth", e);
         src = out;
     }
-    cliffs::k_filter_raise<<<blocks, 256, 0, s>>>(src, out, N, min_depth);
+    cliffs::k_filter_raise<<<blocks, 256, 0, s>>>(src, out, N, min_depth, changed);
     int made = 0;
     e = cliffs::run_filter(out, tmp, nx, ny, alpha, changed, s, &made);
     if (e != cudaSuccess) return fail(CLIFFS_ERR_CUDA, "filter passes", e);

@@ -11,7 +11,7 @@ import pytest
 
 import oracle
 import workloads
-from paper_1410_0753_gb300 import CliffsError, CliffsGrid
+from paper_1410_0753_gb300 import CliffsError, CliffsGrid, cliffs_depth_filter_noalloc
 
 pytestmark = pytest.mark.gpu
 
@@ -285,3 +285,23 @@ def test_depth_filter_of_a_line_of_many_rows():
     g.close()
     want, _ = oracle.depth_filter(d, 2.0, 0.1)
     assert not np.array_equal(want, d) and np.array_equal(got, want)
+
+
+def test_depth_filter_of_a_smooth_depth_stops_early():
+    """A depth that needs no filtering (one pass) takes a fraction of the time of rough relief of the
+    same size (six passes): the library does not launch passes long past the last one needed."""
+    import torch
+    n = 200
+    out = torch.empty(n, n, dtype=torch.float64, device="cuda")
+    times = []
+    for d in (np.full((n, n), 1000.0), 300.0 * np.exp(np.random.default_rng(5).normal(0, 1.0, (n, n))) - 100.0):
+        t = torch.as_tensor(d, device="cuda")
+        runs = []
+        for _ in range(40):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            passes = cliffs_depth_filter_noalloc(t, out, n, n)
+            runs.append(time.perf_counter() - t0)
+        times.append((passes, sorted(runs)[20]))
+    assert times[0][0] == 1 and times[1][0] == 6
+    assert times[0][1] <= 0.45 * times[1][1], times

@@ -1489,12 +1489,13 @@ int cliffs_step_n(cliffs_grid* g, int64_t n) {
         ~CopyBack() { run(); }
     } back{g, rec_state, in_record ? g->step : -1};
     const double t_end = g->bnd_any ? bnd_end(g) : 1e300;
-    // 1D lines: all the steps in one launch (at most LINE_STEPS, some tens of milliseconds),
-    // except one step alone, lines too long for a block, boundary input, timed launches and the
-    // spherical source term of a line along y
+    // 1D lines: all the steps in one launch (at most LINE_STEPS, some tens of milliseconds) where
+    // that is the faster way, except with boundary input, timed launches and the spherical source
+    // term of a line along y
     const long long LINE_STEPS = 65536;
-    if (g->kind != 0 && n > 1 && !g->timing && !g->bnd_any && line_fits(g->kind == 1 ? g->nx : g->ny) &&
-        !(g->kind == 2 && g->cfg.coords != 1)) {
+    if (g->kind != 0) fill_step_args(g, a, 0, 1);
+    if (g->kind != 0 && !g->timing && !g->bnd_any && !(g->kind == 2 && g->cfg.coords != 1) &&
+        line_pays(a, g->B, n, g->kind == 2)) {
         BatchArgs b{};
         for (int i = 0; i < 2; ++i) b.eta[i] = g->eta[i];
         b.emax = g->emax;
@@ -1502,7 +1503,6 @@ int cliffs_step_n(cliffs_grid* g, int64_t n) {
         b.gout = g->cfg.gout;
         b.grec = g->G ? g->grec : nullptr;
         b.grec_row = (long long)g->G * 3;
-        fill_step_args(g, a, 0, 1);
         a.samp = g->items_d;
         for (; n > 0; n -= std::min(n, (int64_t)LINE_STEPS)) {
             const long long m = std::min((long long)n, LINE_STEPS);

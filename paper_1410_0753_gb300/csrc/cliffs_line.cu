@@ -4,6 +4,8 @@
 // the state, depth, metric and maxima: 48 bytes per node, so up to about 4700 nodes), each
 // warp 56 nodes at a time with the x-sweep of the other kernels (the same bits), one block
 // barrier per step. What bounds it is the latency of one sweep, about 0.5 us.
+#include <algorithm>
+
 #include "step_kernels.cuh"
 
 namespace cliffs {
@@ -107,25 +109,58 @@ k_line(const __grid_constant__ StepArgs a, const __grid_constant__ BatchArgs B, 
     if (bad) atomicOr(a.err, ERRF_NONFINITE);
 }
 
-bool line_fits(int nodes) { return (size_t)line_floats(nodes) * LINE_ARRAYS * 4 <= (size_t)LINE_MAX_SMEM; }
-
-cudaError_t launch_line(const StepArgs& a, const BatchArgs& b, int batch, long long step0, long long n, int nsamp,
-                        int along_y, cudaStream_t s) {
+static int line_smem(int nodes) { return line_floats(nodes) * LINE_ARRAYS * 4; }
+static int line_threads(int nodes) { return 32 * std::min(32, (nodes + XOUT - 1) / XOUT); }
+static const void* line_kernel(const StepArgs& a) {
     static const void* const t[8] = {(const void*)k_line<false, false, false>, (const void*)k_line<true, false, false>,
                                      (const void*)k_line<false, true, false>, (const void*)k_line<true, true, false>,
                                      (const void*)k_line<false, false, true>, (const void*)k_line<true, false, true>,
                                      (const void*)k_line<false, true, true>, (const void*)k_line<true, true, true>};
-    const int N = along_y ? a.ny : a.nx, smem = line_floats(N) * LINE_ARRAYS * 4;
-    const void* k = t[(a.K.fric ? 1 : 0) + (a.K.inv_dt2 > 0.f ? 2 : 0) + (a.open_edges ? 4 : 0)];
-    // always the maximum, not this line's size: the attribute belongs to the kernel, and another
-    // thread may launch it for a longer line between these two calls
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, LINE_MAX_SMEM);
+    return t[(a.K.fric ? 1 : 0) + (a.K.inv_dt2 > 0.f ? 2 : 0) + (a.open_edges ? 4 : 0)];
+}
+// always the maximum, not this line's size: the attribute belongs to the kernel, and another
+// thread may launch it for a longer line between this call and the launch
+static cudaError_t optin(const void* k) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, LINE_MAX_SMEM);
+}
+
+// Whether n steps in one launch are faster than n launches. Along y always (a launch of the y-sweep
+// takes 46 us and more). Along x a launch takes 4.2 us and 7 ns per 1000 nodes of the batch (8 with
+// open edges or eq. (solver1)); one launch for all costs 3 us more than a small one and goes in rounds
+// of the blocks that fit on the GPU at once, each loading its line and then passing over it with up
+// to 32 warps at a time, n times.
+// The constants are fitted to 60 .. 4600 nodes, batches of 1 .. 3000 and 2 .. 40 steps; us of a call
+// by launches and in one: 613 nodes x 40 steps 176 and 55, 4600 x 40 176 and 139, x 4 33 and 38, with
+// open edges x 40 178 and 225; 3000 lines of 1000 nodes x 40 986 and 965, with open edges 1160 and 1579.
+bool line_pays(const StepArgs& a, int batch, long long n, int along_y) {
+    const int N = along_y ? a.ny : a.nx;
+    if (!((size_t)line_smem(N) <= (size_t)LINE_MAX_SMEM) || n < 2) return false;
+    if (along_y) return true;
+    int dev = 0, sms = 1, per_sm = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const void* k = line_kernel(a);
+    if (batch > sms && (optin(k) != cudaSuccess || cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                                                       &per_sm, k, line_threads(N), line_smem(N)) != cudaSuccess))
+        return false;
+    const long long at_once = (long long)sms * std::max(1, per_sm), rounds = (batch + at_once - 1) / at_once;
+    const bool s1 = a.K.inv_dt2 > 0.f, open = a.open_edges != 0;
+    const double kn = 1e-3 * N;
+    const double pass = 0.75 + (open ? 0.3 : 0.0) + kn * (0.47 + (s1 ? 0.19 : 0.0) + (open ? 0.40 : 0.0) + (s1 && open ? 0.14 : 0.0));
+    const double step = 4.2 + kn * batch * (s1 || open ? 8e-3 : 7e-3);
+    return 3.0 + (double)rounds * (1.7 + 1.34 * kn + (double)n * pass) < (double)n * step;
+}
+
+cudaError_t launch_line(const StepArgs& a, const BatchArgs& b, int batch, long long step0, long long n, int nsamp,
+                        int along_y, cudaStream_t s) {
+    const int N = along_y ? a.ny : a.nx;
+    const void* k = line_kernel(a);
+    const cudaError_t e = optin(k);
     if (e != cudaSuccess) return e;
     StepArgs aa = a;
     BatchArgs bb = b;
     void* args[] = {&aa, &bb, &step0, &n, &nsamp, &along_y};
-    const int warps = (N + XOUT - 1) / XOUT;
-    return cudaLaunchKernel(k, dim3(batch), dim3(32 * (warps < 32 ? warps : 32)), args, smem, s);
+    return cudaLaunchKernel(k, dim3(batch), dim3(line_threads(N)), args, line_smem(N), s);
 }
 
 }  // namespace cliffs

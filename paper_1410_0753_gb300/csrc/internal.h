@@ -160,7 +160,8 @@ cudaError_t launch_batch_tile(const StepArgs& a, const BatchArgs& b, int blocks,
 int tile_warps_per_block();
 int tile_blocks_per_sm(int tile_rows);
 int tile_max_rows();             // the largest tile_rows of which two blocks fit on an SM
-bool line_fits(int nodes);        // a 1D line of this many nodes fits in one block (cliffs_line.cu)
+// n steps of a 1D grid's scenarios: the line fits in one block and one launch is the faster way (cliffs_line.cu)
+bool line_pays(const StepArgs& a, int batch, long long n, int along_y);
 // steps step0 + 1 .. step0 + n of a 1D grid's scenarios, the samples in a.samp
 cudaError_t launch_line(const StepArgs& a, const BatchArgs& b, int batch, long long step0, long long n, int nsamp,
                         int along_y, cudaStream_t s);

@@ -305,3 +305,24 @@ def test_depth_filter_of_a_smooth_depth_stops_early():
         times.append((passes, sorted(runs)[20]))
     assert times[0][0] == 1 and times[1][0] == 6
     assert times[0][1] <= 0.45 * times[1][1], times
+
+
+@pytest.mark.parametrize("batch,steps", [(1, 200), (1500, 2)])
+def test_lines_take_the_faster_way(batch, steps):
+    """Lines with open edges just short enough for the run in one launch, against lines a little
+    longer, which go by a launch per step: where that way is the faster one, both take it."""
+    times = []
+    for n in (4600, 4900):
+        x = 100.0 * np.arange(n)
+        g = CliffsGrid(n, 1, 1.5, batch=batch, manning_n2=6e-4, open_edges=3, maxout=1 << 30, gout=1 << 20)
+        g.set_bathy(x, np.zeros(1), np.full((1, n), 100.0), False)
+        eta = np.exp(-((x - x[n // 3]) / 5e3) ** 2).astype(np.float32)
+        g.set_initial(np.ascontiguousarray(np.broadcast_to(eta, (batch, 1, n))))
+        runs = []
+        for _ in range(20):
+            t = time.perf_counter()
+            g.step(steps)
+            runs.append(time.perf_counter() - t)
+        times.append(sorted(runs)[5])
+        g.close()
+    assert times[0] <= 1.12 * times[1], times

@@ -109,7 +109,7 @@ k_line(const __grid_constant__ StepArgs a, const __grid_constant__ BatchArgs B, 
     if (bad) atomicOr(a.err, ERRF_NONFINITE);
 }
 
-static int line_smem(int nodes) { return line_floats(nodes) * LINE_ARRAYS * 4; }
+static size_t line_smem(int nodes) { return (size_t)line_floats(nodes) * LINE_ARRAYS * 4; }
 static int line_threads(int nodes) { return 32 * std::min(32, (nodes + XOUT - 1) / XOUT); }
 static const void* line_kernel(const StepArgs& a) {
     static const void* const t[8] = {(const void*)k_line<false, false, false>, (const void*)k_line<true, false, false>,
@@ -134,7 +134,7 @@ static cudaError_t optin(const void* k) {
 // open edges x 40 178 and 225; 3000 lines of 1000 nodes x 40 986 and 965, with open edges 1160 and 1579.
 bool line_pays(const StepArgs& a, int batch, long long n, int along_y) {
     const int N = along_y ? a.ny : a.nx;
-    if (!((size_t)line_smem(N) <= (size_t)LINE_MAX_SMEM) || n < 2) return false;
+    if (line_smem(N) > (size_t)LINE_MAX_SMEM || n < 2) return false;
     if (along_y) return true;
     int dev = 0, sms = 1, per_sm = 1;
     cudaGetDevice(&dev);

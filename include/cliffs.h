@@ -255,7 +255,8 @@ int cliffs_adjoint_recorded_scenario(cliffs_grid* g, int32_t scenario, int32_t c
  * the store grows as the run does), so that cliffs_adjoint_recorded needs no checkpoint pass
  * of its own. A later cliffs_set_initial starts a new record with the same spacing; K = 0
  * stops recording and frees the store. A recording grid runs through cliffs_step_n only (the
- * persistent run rejects it). On a batched grid every scenario is recorded
+ * persistent run rejects it). What is written through cliffs_state_ptrs during a recorded run is
+ * what the next step starts from; the record keeps each state as it was computed. On a batched grid every scenario is recorded
  * (cliffs_adjoint_recorded_scenario). Errors: ERR_STATE before set_initial or after steps
  * since it; ERR_ARG (K < 0, 1D grid). */
 int cliffs_adjoint_record(cliffs_grid* g, int32_t checkpoint_every);
@@ -289,14 +290,16 @@ int cliffs_autotune(cliffs_grid* g, int trials, int32_t* cand, double* us, int32
 
 /* Set the tile shape of the 2D step kernel directly: `rows` output rows per warp (what
  * cliffs_autotune chooses by measurement), e.g. to repeat a measured configuration. Call it
- * after cliffs_set_bathy, which chooses a default shape. Results do not depend on the shape.
+ * after cliffs_set_bathy, which chooses a default shape. Results do not depend on the shape; more
+ * than 512 rows count as 512.
  * Errors: ERR_STATE before set_bathy; ERR_ARG (1D grid, rows outside 1..8192); ERR_NOMEM;
  * ERR_CUDA. */
 int cliffs_set_rows_per_warp(cliffs_grid* g, int32_t rows);
 
 /* Fault injection for tests of the bounded waits (no counterpart in the paper): the next
  * step launch of a 2D grid makes every shared-memory ring slot expect 16 bytes more than
- * its copies deliver, with waits limited to `cycles` clock cycles. Each wait then expires,
+ * its copies deliver (a persistent run that steps by tiles, which have no ring: its grid barrier
+ * one arrival more than it has blocks), with waits limited to `cycles` clock cycles. Each wait then expires,
  * the kernel drains its copies (bounded), sets the timeout flag and returns; later launches
  * of the same call return at once; cliffs_step_n returns CLIFFS_ERR_TIMEOUT and the grid
  * stays usable (its state is whatever the interrupted step left). The injection applies to

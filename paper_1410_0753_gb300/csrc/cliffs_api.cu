@@ -358,7 +358,7 @@ struct cliffs_grid {
     std::vector<int> strip_slow;             // per strip: how many such rows
     ItemSet march, tile;                     // work items of the fused kernel (1D: samples only) and of the tiles
     ItemSet batch;                           // and of the persistent run by marching warps, made when first needed
-    int tile_R = 0, tile_rows = 0;           // rows per tile in open water; the largest tile with its halo
+    int tile_rows = 0;                       // rows of the largest tile, its halo included
     bool S_set = false;                      // S was set or tuned by the caller: steps march
     // timing
     bool timing = false;
@@ -566,7 +566,6 @@ int set_rows_per_warp(cliffs_grid* g, int S) {
 
 int set_tile_rows(cliffs_grid* g, int R) {
     cut_items(g, R, TILE_SLOW, g->tile.items);
-    g->tile_R = R;
     g->tile_rows = 0;
     for (const int4& it : g->tile.items) g->tile_rows = std::max(g->tile_rows, it.z - it.y + 6);
     return upload_items(g, g->tile);

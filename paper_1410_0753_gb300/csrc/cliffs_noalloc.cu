@@ -15,10 +15,10 @@
 
 namespace {
 
-// The scratch every device that loads the library keeps until exit: the first 256 bytes
+// The scratch every device that loads the library keeps until exit: the first 512 bytes
 // hold the passes' "changed" flags, the rest one FP64 Jacobi buffer of up to
 // CLIFFS_NOALLOC_MAX_CELLS nodes.
-constexpr int FLAG_SLOTS = 64;   // 512 bytes
+constexpr int FLAG_SLOTS = 64;
 static_assert(FLAG_SLOTS * 2 >= cliffs::FILTER_PASSES, "one int per pass");
 static __device__ __align__(256) double g_scratch[FLAG_SLOTS + CLIFFS_NOALLOC_MAX_CELLS];
 

@@ -672,9 +672,10 @@ __device__ __forceinline__ bool grid_sync(unsigned long long* bar, unsigned nblo
 // Steps ctl[0]+1 .. ctl[1] of a batch of scenarios in one launch. Scenarios are taken in
 // decreasing order of duration, so those still running at a step are the first nact[step]
 // of `order`; the step's (scenario, item) pairs are numbered scenario-major and warp w of W
-// takes numbers w, w + W, .. (items cost the same, see cut_items; handing them out by an
-// atomic counter put a round trip to L2 before every item, and on small grids queued every
-// warp at one address), then the warps meet at the grid barrier before the next step reads
+// takes numbers w, w + W, .. (cut_items makes items cost about the same; where W is a multiple
+// of the items of a scenario, a warp draws the same item of every scenario, and one with a shore
+// stays the dearer one. Handing them out by an atomic counter put a round trip to L2 before every
+// item, and on small grids queued every warp at one address), then the warps meet at the grid barrier before the next step reads
 // what this one wrote. A scenario that has stopped keeps its last state in the buffer of its
 // last step's parity.
 // With ALT (the alternating order) the odd-indexed steps (st - 1 odd) sweep y first: a second
